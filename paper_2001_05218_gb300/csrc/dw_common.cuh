@@ -874,7 +874,7 @@ __device__ __forceinline__ int block_system(const Batch& B, int b) {
 }
 
 // Per-column (system, right-hand side) CG state, in device memory.
-struct ColState {
+struct alignas(16) ColState {
   double gamma;    // |z|^2, z = A-side residual
   double alpha, beta;
   float alpha_f, beta_f;  // alpha and beta rounded to FP32 by the finalizer
@@ -907,7 +907,7 @@ struct Flags {
   int loops;        // iterations run by the device-driven loop
   int max_loops;    // hard cap on loops (maxiter + 2)
   int rel_runs;     // reliable-update passes run by the device-driven loop
-  int pad;
+  int fin_count;    // columns that the running k_finish has finished (0 between launches)
 };
 
 enum Fin {
@@ -926,7 +926,7 @@ enum Fin {
 };
 
 struct RedArgs {
-  double* partial;
+  DF* partial;
   ColState* cols;
   Flags* flags;
   int fin;
@@ -946,9 +946,8 @@ __device__ __forceinline__ void deactivate(ColState& C, Flags* F, int status) {
   }
 }
 
-// CG scalar recurrences, run by one thread of the last block of a system.
-__device__ __forceinline__ void finalize(const RedArgs& ra, int col, double v) {
-  ColState& C = ra.cols[col];
+// CG scalar recurrences on one column's state, run by one thread.
+__device__ __forceinline__ void finalize(const RedArgs& ra, ColState& C, double v) {
   switch (ra.fin) {
     case FIN_STORE0: C.store[0] = v; break;
     case FIN_STORE1: C.store[1] = v; break;
@@ -1051,7 +1050,8 @@ __device__ __forceinline__ double warp_sum_lane0(double v) {
 
 // Value reduced inside a block: double-float for FP32 and double-float
 // arithmetic (added on the FP32 pipes, about 48 significant bits), IEEE FP64
-// for FP64 arithmetic.  Block partials and both grid levels are IEEE FP64.
+// for FP64 arithmetic.  Block partials are double-float (what the finishing
+// kernel sums in: no conversion on either side); its total is IEEE FP64.
 template <typename R>
 struct RedT {
   using type = DF;
@@ -1063,8 +1063,8 @@ struct RedT<double> {
 __device__ __forceinline__ DF to_red(float v) { return df_make(v, 0.f); }
 __device__ __forceinline__ DF to_red(DF v) { return v; }
 __device__ __forceinline__ double to_red(double v) { return v; }
-__device__ __forceinline__ double red_double(DF v) { return (double)v; }
-__device__ __forceinline__ double red_double(double v) { return v; }
+__device__ __forceinline__ DF to_partial(DF v) { return v; }
+__device__ __forceinline__ DF to_partial(double v) { return DF(v); }
 __device__ __forceinline__ DF red_zero(DF) { return df_make(0.f, 0.f); }
 __device__ __forceinline__ double red_zero(double) { return 0.0; }
 // warp total in lane 0, fixed order, double-float on the FP32 pipes
@@ -1110,7 +1110,7 @@ __device__ __forceinline__ void reduce_block(const SysDesc& S, int T, int RB, in
     if (r < S.nrhs) {
       V s = wpart[tid * wpr];
       for (int w = 1; w < wpr; ++w) s = s + wpart[tid * wpr + w];
-      ra.partial[S.part0 + r * ntiles + tile] = red_double(s);
+      ra.partial[S.part0 + r * ntiles + tile] = to_partial(s);
     }
   }
   store();
@@ -1136,56 +1136,81 @@ __device__ __forceinline__ void reduce_block_n(const SysDesc& S, int T, int RB, 
     if (r < S.nrhs) {
       V s = wpart[j][g * wpr];
       for (int w = 1; w < wpr; ++w) s = s + wpart[j][g * wpr + w];
-      ra.partial[S.part0 + r * ntiles + tile] = red_double(s);
+      ra.partial[S.part0 + r * ntiles + tile] = to_partial(s);
     }
   }
   store();
 }
 
-// Finishing kernel: one block (kFinishThreads threads) per column (system,
-// right-hand side).  Thread t sums partials t, t + kFinishThreads, ... in
-// order (double-float), loading eight at a time so that their L2 round trips
-// overlap, then a fixed warp tree and a fixed sum over warps; thread 0 runs
-// the finalizer in IEEE FP64.  Columns whose kernel was gated off hold stale
-// partials; the finalizer ignores them by the same state the gate tested
-// (active, do_rel, xzero).
-constexpr int kFinishThreads = 1024;
-static __global__ void __launch_bounds__(kFinishThreads) k_finish(const __grid_constant__ Batch B, int par_mode,
-                                                           RedArgs ra) {
+// Where each column's partials lie: what k_finish needs of a Batch.
+struct FinPlan {
+  int nrhs;
+  int part0[kMaxSys], ntiles[kMaxSys];
+};
+
+// Finishing kernel: one block per column (system, right-hand side).  Thread t
+// sums partials t, t + blockDim, ... in order (double-float), loading eight at
+// a time so that their L2 round trips overlap, then a fixed warp tree and a
+// fixed tree over the warps; thread 0 runs the finalizer in IEEE FP64.
+// Columns whose kernel was gated off hold stale partials; the finalizer
+// ignores them by the same state the gate tested (active, do_rel, xzero).
+//
+// The kernel is one serial chain of latencies, so it is kept short: the
+// column's state is loaded beside the partials and written back whole, the
+// warps' sums meet in a shuffle tree, and up to 2048 partials take 256 threads
+// instead of 1024 (launching and draining 32 warps costs more than a longer
+// loop).  With rel.on the last column to finish also sets the condition of the
+// reliable-update node (a separate one-thread kernel would cost about 2 us).
+// Measured at 16^3x32 (512 partials): 4.2 us per launch before, see k_finish's
+// caller for the rule on the block size.
+constexpr int kFinishThreads = 1024, kFinishThreadsSmall = 256;
+struct RelCond {
+  unsigned long long handle;
+  int on;
+};
+static __global__ void __launch_bounds__(kFinishThreads) k_finish(const __grid_constant__ FinPlan F, RedArgs ra,
+                                                                  RelCond rel) {
   __shared__ DF wpart[kFinishThreads / 32];
   const int col = blockIdx.x;
-  const int nrhs = B.sd[0].nrhs;
-  const int si = col / nrhs, r = col - si * nrhs;
-  const SysDesc& S = B.sd[si];
-  const int ntiles = par_mode == 2 ? 2 * S.tpp : S.tpp;
-  const double* p = ra.partial + S.part0 + (size_t)r * ntiles;
+  const int si = F.nrhs == 1 ? col : col / F.nrhs, r = col - si * F.nrhs;
+  const int ntiles = F.ntiles[si];
+  const DF* p = ra.partial + F.part0[si] + (size_t)r * ntiles;
+  ColState C;
+  if (threadIdx.x == 0) C = ra.cols[col];
   DF v = df_make(0.f, 0.f);
-  for (int i0 = threadIdx.x; i0 < ntiles; i0 += 8 * kFinishThreads) {
-    double t[8];
+  for (int i0 = threadIdx.x; i0 < ntiles; i0 += 8 * blockDim.x) {
+    float2 t[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-      const int i = i0 + j * kFinishThreads;
-      t[j] = i < ntiles ? __ldcg(p + i) : 0.0;
+      const int i = i0 + j * blockDim.x;
+      t[j] = i < ntiles ? __ldcg(reinterpret_cast<const float2*>(p + i)) : make_float2(0.f, 0.f);
     }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v = v + DF(t[j]);
+    for (int j = 0; j < 8; ++j) v = v + df_make(t[j].x, t[j].y);
   }
   v = warp_sum_lane0(v);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0) wpart[warp] = v;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    DF t = wpart[0];
-    for (int w = 1; w < kFinishThreads / 32; ++w) t = t + wpart[w];
-    finalize(ra, S.col0 + r, (double)t);
+  if (warp != 0) return;
+  v = lane < (int)(blockDim.x >> 5) ? wpart[lane] : df_make(0.f, 0.f);
+  v = warp_sum_lane0(v);
+  if (lane != 0) return;
+  finalize(ra, C, (double)v);
+  ra.cols[col] = C;
+  if (rel.on) {
+    bool last = gridDim.x == 1;
+    if (!last) {
+      __threadfence();  // this column's update of rel_pending before its count
+      last = atomicAdd(&ra.flags->fin_count, 1) == (int)gridDim.x - 1;
+    }
+    if (last) {
+      ra.flags->fin_count = 0;
+      const bool run = atomicAdd(&ra.flags->rel_pending, 0) > 0;
+      if (run) ra.flags->rel_runs += 1;
+      cudaGraphSetConditional(rel.handle, run ? 1u : 0u);
+    }
   }
-}
-
-// Cooperative copy of this block's system descriptor into shared memory.
-__device__ __forceinline__ void load_desc(SysDesc& S, const SysDesc* __restrict__ sd, int si) {
-  const int* src = reinterpret_cast<const int*>(sd + si);
-  int* dst = reinterpret_cast<int*>(&S);
-  for (int i = threadIdx.x; i < (int)(sizeof(SysDesc) / 4); i += blockDim.x) dst[i] = src[i];
 }
 
 }  // namespace dw

@@ -100,7 +100,9 @@ SolveCacheEntry* solve_cache_insert(SolveCacheEntry&& e);
 
 // The second kernel of a grid reduction: sums the partials of the kernel just
 // launched (par_mode as that kernel's) per column and runs finalizer fin.
-inline void finish(const Exec& E, int par_mode, int fin) {
+// Up to 2048 partials per column take 256 threads (one round of eight loads
+// each), more take 1024.
+inline void finish(const Exec& E, int par_mode, int fin, RelCond rel = RelCond{0, 0}) {
   Profiler& pr = profiler();
   cudaEvent_t ea = nullptr, eb = nullptr;
   if (pr.on) pr.launches += 1;
@@ -109,7 +111,17 @@ inline void finish(const Exec& E, int par_mode, int fin) {
     eb = pr.event();
     cudaEventRecord(ea, E.st);
   }
-  k_finish<<<E.P.ncols, kFinishThreads, 0, E.st>>>(E.P.B, par_mode, E.ra(fin));
+  FinPlan F;
+  F.nrhs = E.P.nrhs;
+  int most = 0;
+  for (int i = 0; i < kMaxSys; ++i) {
+    const SysDesc& S = E.P.B.sd[i];
+    F.part0[i] = i < E.P.nsys ? S.part0 : 0;
+    F.ntiles[i] = i < E.P.nsys ? (par_mode == 2 ? 2 * S.tpp : S.tpp) : 0;
+    if (F.ntiles[i] > most) most = F.ntiles[i];
+  }
+  const int threads = most <= 8 * kFinishThreadsSmall ? kFinishThreadsSmall : kFinishThreads;
+  k_finish<<<E.P.ncols, threads, 0, E.st>>>(F, E.ra(fin), rel);
   if (pr.timing) {
     cudaEventRecord(eb, E.st);
     Profiler::Rec r;

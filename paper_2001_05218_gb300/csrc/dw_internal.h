@@ -77,7 +77,7 @@ struct Plan {
   Batch B;
   int pair = 0;      // 16-bit Wilson stencils: two right-hand sides per thread (k_hop_pair)
   int nsys = 0, nrhs = 1, ncols = 0;
-  int partials = 0;  // doubles in the partial-sum buffer (one per block and column)
+  int partials = 0;  // values in the partial-sum buffer (one per block and column)
   dim3 block, grid1, grid2;  // one parity / both parities
 };
 // T sites per block and RB right-hand sides per block (T*RB <= 256, T a
@@ -103,7 +103,7 @@ std::string tune_key(const dw_lattice* lats, int n, int nrhs, int prec, int c12)
 
 // Device scratch for reductions of one plan.
 struct RedBuf {
-  double* partial = nullptr;
+  DF* partial = nullptr;
   ColState* cols = nullptr;
   Flags* flags = nullptr;
 };

@@ -634,40 +634,37 @@ struct EpiResidFull {
 };
 
 // ------------------------------------------------------------------ block prologue
-// System descriptor into shared memory, the gate of every column of the
-// system, this thread's site s on output parity par and right-hand side r.
-// A block returns at once only when every column of its system is gated off:
-// all blocks of a system read the same gates (they change only in the
-// system's last block, after every block has read them), so either all of a
-// system's blocks arrive at the reduction or none does.
+// This block's system descriptor S, this thread's site s on output parity par,
+// its right-hand side r, and whether it has work (valid): in range and its
+// column's gate open.  The descriptor is read where it is used, from the
+// kernel parameter in the constant bank, and every thread tests its own gate:
+// no copy, no barrier and one global load ahead of a thread's first operand
+// load.  (A copy of the descriptor in shared memory, a barrier, the gates of
+// all columns and a second barrier held every block's SM slot for about 1 us
+// before its first load.)  The reduction needs no agreement between blocks on
+// a gate: a closed column's partials are ignored by its finalizer.
 #define DW_BLOCK_PROLOGUE(GATE)                                            \
-  __shared__ SysDesc S;                                                    \
-  __shared__ int act[64];                                                  \
   const int T = B.T, RB = B.RB;                                            \
   /* the right-hand-side block varies fastest: the blocks of one tile run  \
      together and share its links and neighbours in L2 */                  \
   const unsigned bx_ = B.rev ? gridDim.x - 1u - blockIdx.x : blockIdx.x;   \
-  const int by = (int)(bx_ % (unsigned)B.ny);                              \
-  int b = (int)(bx_ / (unsigned)B.ny), par;                                \
+  int by = 0, b = (int)bx_, par, rl = 0;                                   \
+  if (B.ny > 1) {                                                          \
+    b = (int)(bx_ / (unsigned)B.ny);                                       \
+    by = (int)bx_ - b * B.ny;                                              \
+  }                                                                        \
   if (par_mode == 2) {                                                     \
     par = b >= B.ntot ? 1 : 0;                                             \
     b -= par * B.ntot;                                                     \
   } else {                                                                 \
     par = par_mode;                                                        \
   }                                                                        \
-  load_desc(S, B.sd, block_system(B, b));                                  \
-  __syncthreads();                                                         \
-  for (int i_ = threadIdx.x; i_ < S.nrhs; i_ += blockDim.x)                \
-    act[i_] = gate_of(GATE, ra.cols, S.col0 + i_);                         \
-  __syncthreads();                                                         \
-  int any = 0;                                                             \
-  for (int i_ = 0; i_ < S.nrhs; ++i_) any |= act[i_];                      \
-  if (!any) return;                                                        \
-  const int rl = threadIdx.x / T;                                          \
+  const SysDesc& S = B.sd[block_system(B, b)];                             \
+  if (RB > 1) rl = (int)threadIdx.x / T;                                   \
   const int r = by * RB + rl;                                              \
   const int tile = b - S.tile0;                                            \
-  const int s = tile * T + (threadIdx.x - rl * T);                         \
-  const bool valid = s < S.vh && r < S.nrhs && act[r < S.nrhs ? r : 0];
+  const int s = tile * T + ((int)threadIdx.x - rl * T);                    \
+  const bool valid = s < S.vh && r < S.nrhs && gate_of(GATE, ra.cols, S.col0 + r);
 
 #define DW_BLOCK_REDUCE(val)                                               \
   {                                                                        \
@@ -912,8 +909,6 @@ template <int SPA, bool C12, bool DAG, class Epi>
 __global__ void __launch_bounds__(256, 2)
     k_hop_pair(const __grid_constant__ Batch B, int par_mode, int link_slot, int in_slot, Epi epi, RedArgs ra) {
   static_assert(SPA == P16 || SPA == PB16, "two right-hand sides per thread: 16-bit storage");
-  __shared__ SysDesc S;
-  __shared__ int act[64];
   const int T = B.T, RB = B.RB;
   const unsigned ny = (unsigned)((B.sd[0].nrhs + 2 * RB - 1) / (2 * RB));
   const unsigned bx = B.rev ? gridDim.x - 1u - blockIdx.x : blockIdx.x;
@@ -925,20 +920,14 @@ __global__ void __launch_bounds__(256, 2)
   } else {
     par = par_mode;
   }
-  load_desc(S, B.sd, block_system(B, b));
-  __syncthreads();
-  for (int i_ = threadIdx.x; i_ < S.nrhs; i_ += blockDim.x) act[i_] = gate_of(epi.gate, ra.cols, S.col0 + i_);
-  __syncthreads();
-  int any = 0;
-  for (int i_ = 0; i_ < S.nrhs; ++i_) any |= act[i_];
-  if (!any) return;
+  const SysDesc& S = B.sd[block_system(B, b)];
   const int rl = threadIdx.x / T;
   const int r0 = (by * RB + rl) * 2, r1 = r0 + 1;
   const int tile = b - S.tile0;
   const int s = tile * T + (threadIdx.x - rl * T);
   const bool site = s < S.vh;
-  const bool v0 = site && r0 < S.nrhs && act[r0 < S.nrhs ? r0 : 0];
-  const bool v1 = site && r1 < S.nrhs && act[r1 < S.nrhs ? r1 : 0];
+  const bool v0 = site && r0 < S.nrhs && gate_of(epi.gate, ra.cols, S.col0 + r0);
+  const bool v1 = site && r1 < S.nrhs && gate_of(epi.gate, ra.cols, S.col0 + r1);
   const int r1l = r1 < S.nrhs ? r1 : r0;  // a missing second column reloads the first
   typename RedT<float>::type nrm[2] = {red_zero(typename RedT<float>::type()), red_zero(typename RedT<float>::type())};
   typename Epi::Packed po0, po1;
@@ -1038,10 +1027,24 @@ __global__ void __launch_bounds__(256) k_update_r(const __grid_constant__ Batch 
   })
 }
 
+// The while-node condition set by the loop's last kernel (on = 0: no loop).
+struct LoopCond {
+  unsigned long long handle;
+  int on;
+};
+
 // xl += alpha_x p (the increment of the iteration that used p, unless a
 // reliable update has folded it already: alpha_x = 0);  p = z + beta p
 template <int SPL, int SPA>
-__global__ void __launch_bounds__(256) k_update_p(const __grid_constant__ Batch B, int par_mode, RedArgs ra) {
+__global__ void __launch_bounds__(256) k_update_p(const __grid_constant__ Batch B, int par_mode, RedArgs ra,
+                                                  LoopCond lc) {
+  // last kernel of an iteration: decides whether the device-driven loop goes on
+  // (no kernel of its own: a one-thread node costs about 2 us per iteration)
+  if (lc.on && blockIdx.x == 0 && threadIdx.x == 0) {
+    const int loops = ra.flags->loops + 1;
+    ra.flags->loops = loops;
+    cudaGraphSetConditional(lc.handle, (ra.flags->active > 0 && loops < ra.flags->max_loops) ? 1u : 0u);
+  }
   DW_BLOCK_PROLOGUE(G_ACTIVE)
   if (valid) {
     using RL = typename Spin<SPL>::R;

@@ -23,14 +23,14 @@ extern "C" dw_status dw_apply_norm(const dw_field* U, const dw_field* in, dw_fie
   auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
   const size_t tmp_b =
       in->kind == DW_SPINOR_FULL ? 0 : al((size_t)in->nrhs * spin_bytes(in->prec) * vh_of(in->lat));
-  const size_t part_b = al(sizeof(double) * E.P.partials);
+  const size_t part_b = al(sizeof(DF) * E.P.partials);
   const size_t cols_b = al(sizeof(ColState) * E.P.ncols), flags_b = al(sizeof(Flags));
   char* buf = nullptr;
   DW_CUDA(cudaMallocAsync((void**)&buf, tmp_b + part_b + cols_b + flags_b, st));
   char* p = buf;
   if (tmp_b) S.f[S_AUX1] = arena_slot(p, in->lat, in->prec, in->nrhs, 1);
   p += tmp_b;
-  E.rb.partial = reinterpret_cast<double*>(p);
+  E.rb.partial = reinterpret_cast<DF*>(p);
   p += part_b;
   E.rb.cols = reinterpret_cast<ColState*>(p);
   p += cols_b;

@@ -136,18 +136,6 @@ struct CG {
   static dw_status run_stepped(const Exec& E, int mode, int maxiter);
 };
 
-// Condition setters for the device-driven loop (one thread).
-static __global__ void k_cond_rel(Flags* f, cudaGraphConditionalHandle h) {
-  const bool run = f->rel_pending > 0;
-  if (run) f->rel_runs += 1;
-  cudaGraphSetConditional(h, run ? 1u : 0u);
-}
-static __global__ void k_cond_loop(Flags* f, cudaGraphConditionalHandle h) {
-  const int loops = f->loops + 1;
-  f->loops = loops;
-  cudaGraphSetConditional(h, (f->active > 0 && loops < f->max_loops) ? 1u : 0u);
-}
-
 struct CaptureStreams {
   cudaStream_t a = nullptr, b = nullptr;
   CaptureStreams() {
@@ -157,7 +145,8 @@ struct CaptureStreams {
 };
 
 // The whole CG loop as one graph: while (active columns) { iteration with the
-// reliable update in an if-node }.  Both conditions are set on the device,
+// reliable update in an if-node }.  Both conditions are set on the device, by
+// kernels of the iteration (k_finish after the update of r, and k_update_p),
 // the loop is capped at maxiter + 2 passes, and every column also leaves the
 // loop through its own maxiter / timeout / breakdown checks.
 template <int L, int A, bool C12, int H, int OP>
@@ -193,10 +182,8 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, int mode, cudaGraphE
   DW_CUDA(cudaStreamBeginCaptureToGraph(cs.a, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
   wstep(E, mode);
   count_launch();
-  count_launch();
   k_update_r<L><<<E.grid(pm), E.P.block, 0, E.st>>>(E.P.B, pm, E.ra(FIN_UPDATE));
-  finish(E, pm, FIN_UPDATE);
-  k_cond_rel<<<1, 1, 0, E.st>>>(E.rb.flags, hr);
+  finish(E, pm, FIN_UPDATE, RelCond{(unsigned long long)hr, 1});
   {
     cudaStreamCaptureStatus cst;
     cudaGraph_t capg;
@@ -222,9 +209,8 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, int mode, cudaGraphE
     c2 = pr.launches;
   }
   zstep(E, mode, FIN_BETA);
-  k_update_p<L, A><<<E.grid(pm), E.P.block, 0, E.st>>>(E.flipped().batch(), pm, E.ra(FIN_STORE0));
-  k_cond_loop<<<1, 1, 0, E.st>>>(E.rb.flags, hw);
-  count_launch();
+  k_update_p<L, A><<<E.grid(pm), E.P.block, 0, E.st>>>(E.flipped().batch(), pm, E.ra(FIN_STORE0),
+                                                       LoopCond{(unsigned long long)hw, 1});
   count_launch();
   cudaGraph_t tmp;
   DW_CUDA(cudaStreamEndCapture(cs.a, &tmp));
@@ -269,7 +255,7 @@ dw_status CG<L, A, C12, H, OP>::run_stepped(const Exec& E, int mode, int maxiter
     if (hf->active == 0) continue;
     zstep(E, mode, FIN_BETA);
     count_launch();
-    k_update_p<L, A><<<E.grid(pm), E.P.block, 0, E.st>>>(E.flipped().batch(), pm, E.ra(FIN_STORE0));
+    k_update_p<L, A><<<E.grid(pm), E.P.block, 0, E.st>>>(E.flipped().batch(), pm, E.ra(FIN_STORE0), LoopCond{0, 0});
   }
   DW_CUDA(cudaGetLastError());
   return DW_OK;
@@ -350,11 +336,11 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
         total += al((size_t)nrhs * pc.npar * spin_bytes(pc.prec) * vh);
       }
     }
-    const size_t red_bytes = al(sizeof(double) * F.P.partials) + al(sizeof(ColState) * F.P.ncols) + al(sizeof(Flags));
+    const size_t red_bytes = al(sizeof(DF) * F.P.partials) + al(sizeof(ColState) * F.P.ncols) + al(sizeof(Flags));
     DW_CUDA(cudaMalloc((void**)&fresh.arena, total + red_bytes));
     char* rp = fresh.arena + total;
-    F.rb.partial = reinterpret_cast<double*>(rp);
-    rp += al(sizeof(double) * F.P.partials);
+    F.rb.partial = reinterpret_cast<DF*>(rp);
+    rp += al(sizeof(DF) * F.P.partials);
     F.rb.cols = reinterpret_cast<ColState*>(rp);
     rp += al(sizeof(ColState) * F.P.ncols);
     F.rb.flags = reinterpret_cast<Flags*>(rp);
@@ -452,7 +438,7 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
   }
   zstep(E, mode, FIN_GAMMA0);  // z, gamma
   count_launch();
-  k_update_p<L, A><<<E.grid(eo ? 0 : 2), E.P.block, 0, st>>>(E.P.B, eo ? 0 : 2, E.ra(FIN_STORE0));  // p = z
+  k_update_p<L, A><<<E.grid(eo ? 0 : 2), E.P.block, 0, st>>>(E.P.B, eo ? 0 : 2, E.ra(FIN_STORE0), LoopCond{0, 0});  // p = z
   DW_CUDA(cudaGetLastError());
 
   // ---- iterations

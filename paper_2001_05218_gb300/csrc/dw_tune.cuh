@@ -55,7 +55,7 @@ BlockShape tune_inner_shape(const std::vector<dw_lattice>& lats, int nrhs, const
   size_t part_b = 0, cols_b = 0;
   for (size_t i = 0; i < cand.size(); ++i) {
     make_plan(plans[i], lats, nrhs, cand[i].T, cand[i].RB);
-    part_b = std::max(part_b, al(sizeof(double) * plans[i].partials));
+    part_b = std::max(part_b, al(sizeof(DF) * plans[i].partials));
     cols_b = std::max(cols_b, al(sizeof(ColState) * plans[i].ncols));
   }
   const size_t red_b = part_b + cols_b + al(sizeof(Flags));
@@ -63,7 +63,7 @@ BlockShape tune_inner_shape(const std::vector<dw_lattice>& lats, int nrhs, const
   if (cudaMallocAsync((void**)&buf, 3 * per + red_b, st) != cudaSuccess) return BlockShape{0, 0};
   cudaMemsetAsync(buf, 0, 3 * per + red_b, st);
   RedBuf rb;
-  rb.partial = reinterpret_cast<double*>(buf + 3 * per);
+  rb.partial = reinterpret_cast<DF*>(buf + 3 * per);
   rb.cols = reinterpret_cast<ColState*>(buf + 3 * per + part_b);
   rb.flags = reinterpret_cast<Flags*>(buf + 3 * per + part_b + cols_b);
   Profiler& pr = profiler();
