@@ -417,6 +417,20 @@ struct Spin<P64> {
   }
   // v <- the value a store followed by a load would give
   __device__ static __forceinline__ void roundtrip(Cx<double> (&)[12]) {}
+  // the three colours of one spin
+  __device__ static __forceinline__ void load_spin(const char* base, int vh, int s, int spin, Cx<double> (&v)[3]) {
+    const double2* b = reinterpret_cast<const double2*>(base) + (size_t)(3 * spin) * vh + s;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      double2 t = __ldg(b + (size_t)c * vh);
+      v[c] = cx(t.x, t.y);
+    }
+  }
+  __device__ static __forceinline__ void store_spin(char* base, int vh, int s, int spin, const Cx<double> (&v)[3]) {
+    double2* b = reinterpret_cast<double2*>(base) + (size_t)(3 * spin) * vh + s;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) b[(size_t)c * vh] = make_double2(v[c].re, v[c].im);
+  }
 };
 
 template <>
@@ -589,13 +603,18 @@ struct Spin<PDF> {
   }
   // the three colours of one spin
   __device__ static __forceinline__ void load_spin(const char* base, int vh, int s, int spin, Cx<DF> (&v)[3]) {
-    const float4* b = reinterpret_cast<const float4*>(base);
+    const float4* b = reinterpret_cast<const float4*>(base) + (size_t)(3 * spin) * vh + s;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      float4 t = __ldg(b + (size_t)(3 * spin + c) * vh + s);
+      float4 t = __ldg(b + (size_t)c * vh);
       v[c].re = df_make(t.x, t.y);
       v[c].im = df_make(t.z, t.w);
     }
+  }
+  __device__ static __forceinline__ void store_spin(char* base, int vh, int s, int spin, const Cx<DF> (&v)[3]) {
+    float4* b = reinterpret_cast<float4*>(base) + (size_t)(3 * spin) * vh + s;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) b[(size_t)c * vh] = make_float4(v[c].re.hi, v[c].re.lo, v[c].im.hi, v[c].im.lo);
   }
   __device__ static __forceinline__ void roundtrip(Cx<DF> (&)[12]) {}
 };

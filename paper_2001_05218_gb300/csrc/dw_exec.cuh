@@ -144,7 +144,15 @@ inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int 
     eb = pr.event();
     cudaEventRecord(ea, E.st);
   }
+  // FP64-class Wilson stencils: two threads per site
+  constexpr bool kRows =
+      (SPA == P64 || SPA == PDF) && LP == SPA && OP == OP_WILSON && std::is_same<In, InOne<SPA>>::value;
   bool launched = false;
+  if constexpr (kRows) {
+    k_hop_rows<SPA, C12, DAG, Epi><<<E.grid(par_mode), 2 * E.P.block.x, 0, E.st>>>(E.batch(), par_mode, link_slot,
+                                                                                  in.slot, epi, E.ra(fin));
+    launched = true;
+  }
   if constexpr ((SPA == P16 || SPA == PB16) && LP == SPA && OP == OP_WILSON && std::is_same<In, InOne<SPA>>::value) {
     if (E.P.pair && E.P.nrhs >= 2) {  // two right-hand sides per thread, each link loaded once for both
       const unsigned npar = par_mode == 2 ? 2u : 1u;
@@ -153,9 +161,10 @@ inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int 
       launched = true;
     }
   }
-  if (!launched)
-    k_hop<SPA, LP, C12, DAG, In, Epi, OP><<<E.grid(par_mode), E.P.block, 0, E.st>>>(E.batch(), par_mode, link_slot, in,
+  if constexpr (!kRows) {
+    if (!launched) k_hop<SPA, LP, C12, DAG, In, Epi, OP><<<E.grid(par_mode), E.P.block, 0, E.st>>>(E.batch(), par_mode, link_slot, in,
                                                                                     epi, E.ra(fin));
+  }
   if (pr.timing) {
     cudaEventRecord(eb, E.st);
     const int npar = par_mode == 2 ? 2 : 1;

@@ -277,83 +277,8 @@ __device__ __forceinline__ void su3_mul(const Cx<DF> (&u)[9], const Cx<DF> (&h)[
 }
 #endif
 
-// Runtime-direction form of the spin projection and reconstruction, used by
-// the double-float stencil whose unrolled body would not fit the instruction
-// cache.  For (1 + s gamma_mu):  h0 = p0 + c0 q0,  h1 = p1 + c1 q1 with
-// (q0, q1) = (p3, p2) for mu = x, y and (p2, p3) for mu = z, t; the lower spins
-// are d2 (g1 or g0) and d3 (g0 or g1) with the same pairing.  Every factor is
-// +-1 or +-i:
-//   mu = x: c0 = c1 = -s i;   d2 = d3 = s i
-//   mu = y: c0 = -s, c1 = s;  d2 = s, d3 = -s
-//   mu = z: c0 = -s i, c1 = s i; d2 = s i, d3 = -s i
-//   mu = t: c0 = c1 = s;      d2 = d3 = s
-struct UnitFactor {
-  bool imag;   // multiply by i
-  bool neg;    // then by -1
-};
-template <typename R>
-__device__ __forceinline__ Cx<R> mul_unit(Cx<R> q, UnitFactor f) {
-  Cx<R> r = f.imag ? cx(-q.im, q.re) : q;
-  return f.neg ? cx(-r.re, -r.im) : r;
-}
-struct DirSpin {
-  bool swap;  // pair spin 0 with spin 3 (x, y)
-  UnitFactor c0, c1, d2, d3;
-};
-__device__ __forceinline__ DirSpin dir_spin(int mu, int s) {
-  DirSpin d;
-  const bool neg_s = s < 0;
-  d.swap = mu <= 1;
-  const bool im = (mu == 0 || mu == 2);
-  d.c0 = UnitFactor{im, mu == 3 ? neg_s : !neg_s};
-  d.c1 = UnitFactor{im, mu == 0 ? !neg_s : neg_s};
-  d.d2 = UnitFactor{im, neg_s};
-  d.d3 = UnitFactor{im, (mu == 1 || mu == 2) ? !neg_s : neg_s};
-  return d;
-}
 // complex sums for the double-float path: lazy (no renormalisation)
 __device__ __forceinline__ Cx<DF> cadd_lazy(Cx<DF> a, Cx<DF> b) { return cx(add_lazy(a.re, b.re), add_lazy(a.im, b.im)); }
-template <typename R>
-__device__ __forceinline__ void project_rt(const DirSpin& d, const Cx<R> (&p)[12], Cx<R> (&h)[6]) {
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    const Cx<R> q0 = d.swap ? p[9 + c] : p[6 + c];
-    const Cx<R> q1 = d.swap ? p[6 + c] : p[9 + c];
-    h[c] = cadd_lazy(p[c], mul_unit(q0, d.c0));
-    h[3 + c] = cadd_lazy(p[3 + c], mul_unit(q1, d.c1));
-  }
-}
-// The same projection from a double-float field, loading for each half-spinor
-// row only the two spins it combines, so that six of the twelve components
-// are live at a time.
-template <class In>
-__device__ __forceinline__ void project_rt_loaded(const DirSpin& d, const In& in, const SysDesc& S, int par, int r,
-                                                  int n, Cx<DF> (&h)[6]) {
-  const char* base = slot_ptr(S, in.slot, r, par);
-  Cx<DF> a[3], q[3];
-  Spin<PDF>::load_spin(base, S.vh, n, 0, a);
-  Spin<PDF>::load_spin(base, S.vh, n, d.swap ? 3 : 2, q);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) h[c] = cadd_lazy(a[c], mul_unit(q[c], d.c0));
-  Spin<PDF>::load_spin(base, S.vh, n, 1, a);
-  Spin<PDF>::load_spin(base, S.vh, n, d.swap ? 2 : 3, q);
-#pragma unroll
-  for (int c = 0; c < 3; ++c) h[3 + c] = cadd_lazy(a[c], mul_unit(q[c], d.c1));
-}
-// acc stays unnormalised across the eight directions (renormalised by the caller)
-template <typename R>
-__device__ __forceinline__ void accumulate_rt(const DirSpin& d, Cx<R> (&acc)[12], const Cx<R> (&g)[6]) {
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    acc[c] = cadd_lazy(acc[c], g[c]);
-    acc[3 + c] = cadd_lazy(acc[3 + c], g[3 + c]);
-    const Cx<R> g2 = d.swap ? g[3 + c] : g[c];
-    const Cx<R> g3 = d.swap ? g[c] : g[3 + c];
-    acc[6 + c] = cadd_lazy(acc[6 + c], mul_unit(g2, d.d2));
-    acc[9 + c] = cadd_lazy(acc[9 + c], mul_unit(g3, d.d3));
-  }
-}
-
 // Site coordinates of even-odd index s on parity par.
 struct Coord {
   int xh, x, y, z, t, row;  // row = s - xh (start of the x-row in eo indexing)
@@ -461,11 +386,99 @@ struct InOne {
   }
 };
 
+// ------------------------------------------------------------------ half sites
+// Two threads per site (k_hop_rows): lanes j and j + 16 of a warp hold spins
+// (0, 2) and (1, 3) of one site, a[c] = spin row, b[c] = spin 2 + row.
+__device__ __forceinline__ uint32_t other_row(uint32_t w) { return __shfl_xor_sync(0xffffffffu, w, 16); }
+__device__ __forceinline__ float other_row(float v) { return __shfl_xor_sync(0xffffffffu, v, 16); }
+__device__ __forceinline__ double other_row(double v) { return __shfl_xor_sync(0xffffffffu, v, 16); }
+__device__ __forceinline__ DF other_row(DF v) { return df_make(other_row(v.hi), other_row(v.lo)); }
+template <typename R>
+__device__ __forceinline__ Cx<R> other_row(Cx<R> v) { return cx(other_row(v.re), other_row(v.im)); }
+
+// Store of one site in storage SP by its two threads (all lanes call it; lanes
+// with ok = false take part in the exchanges only).  FP32 and 16-bit planes
+// hold neighbouring complex numbers k = 3 spin + colour side by side, so the
+// rows swap the ones that lie in the other's planes.
+template <int SP, typename R>
+__device__ __forceinline__ void store_rows(char* base, int vh, int s, int row, const Cx<R> (&a)[3],
+                                           const Cx<R> (&b)[3], bool ok) {
+  if constexpr (SP == P64 || SP == PDF) {
+    using RS = typename Spin<SP>::R;
+    Cx<RS> u[3], v[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      u[c] = cx((RS)a[c].re, (RS)a[c].im);
+      v[c] = cx((RS)b[c].re, (RS)b[c].im);
+    }
+    if (ok) {
+      Spin<SP>::store_spin(base, vh, s, row, u);
+      Spin<SP>::store_spin(base, vh, s, 2 + row, v);
+    }
+  } else if constexpr (SP == P32) {
+    Cx<float> u[3], v[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      u[c] = cx((float)a[c].re, (float)a[c].im);
+      v[c] = cx((float)b[c].re, (float)b[c].im);
+    }
+    // row 0 holds k = 0 1 2 | 6 7 8 and stores planes 0 (0 1), 1 (2 3), 3 (6 7);
+    // row 1 holds k = 3 4 5 | 9 10 11 and stores planes 2 (4 5), 4 (8 9), 5 (10 11)
+    const Cx<float> got = other_row(row == 0 ? v[2] : u[0]);  // row 0: k = 3, row 1: k = 8
+    float4* o = reinterpret_cast<float4*>(base) + s;
+    if (ok) {
+      if (row == 0) {
+        o[0] = make_float4(u[0].re, u[0].im, u[1].re, u[1].im);
+        o[(size_t)vh] = make_float4(u[2].re, u[2].im, got.re, got.im);
+        o[(size_t)3 * vh] = make_float4(v[0].re, v[0].im, v[1].re, v[1].im);
+      } else {
+        o[(size_t)2 * vh] = make_float4(u[1].re, u[1].im, u[2].re, u[2].im);
+        o[(size_t)4 * vh] = make_float4(got.re, got.im, v[0].re, v[0].im);
+        o[(size_t)5 * vh] = make_float4(v[1].re, v[1].im, v[2].re, v[2].im);
+      }
+    }
+  } else {
+    Cx<float> u[3], v[3];
+    float m = 0.f;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      u[c] = cx((float)a[c].re, (float)a[c].im);
+      v[c] = cx((float)b[c].re, (float)b[c].im);
+      m = fmaxf(m, fmaxf(fmaxf(fabsf(u[c].re), fabsf(u[c].im)), fmaxf(fabsf(v[c].re), fabsf(v[c].im))));
+    }
+    m = fmaxf(m, other_row(m));
+    m = m >= 1e-30f ? m : 0.f;  // as site_max
+    const float inv = m > 0.f ? 1.0f / m : 0.f;
+    uint32_t p[3], q[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      p[c] = H16<SP>::from2(u[c].re * inv, u[c].im * inv);
+      q[c] = H16<SP>::from2(v[c].re * inv, v[c].im * inv);
+    }
+    // row 0 holds words 0 1 2 | 6 7 8 and stores plane 0 (0-3) and the scale;
+    // row 1 holds words 3 4 5 | 9 10 11 and stores planes 1 (4-7) and 2 (8-11)
+    const uint32_t x0 = other_row(row == 0 ? q[0] : p[0]);  // row 0: word 3, row 1: word 6
+    const uint32_t x1 = other_row(q[1]), x2 = other_row(q[2]);
+    uint4* o = reinterpret_cast<uint4*>(base) + s;
+    if (ok) {
+      if (row == 0) {
+        o[0] = make_uint4(p[0], p[1], p[2], x0);
+        reinterpret_cast<float*>(base + (size_t)48 * vh)[s] = m;
+      } else {
+        o[(size_t)vh] = make_uint4(p[1], p[2], x0, x1);
+        o[(size_t)2 * vh] = make_uint4(x2, q[0], q[1], q[2]);
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------------ epilogues
 // write(): forms and stores the output of one site.  Reducing epilogues with
 // kSplit also offer prepare() (forms the stored words and the reduced value)
 // and commit() (stores them), so that the kernel can publish its block's
-// partial sum before the output stores.
+// partial sum before the output stores.  write_rows() is write() for a site
+// held by two threads (k_hop_rows): a, b are the accumulated spins row and
+// 2 + row; every lane calls it, lanes with ok = false store nothing.
 // out = coef * H in
 template <int SPO, int COEF>
 struct EpiOut {
@@ -483,6 +496,19 @@ struct EpiOut {
 #pragma unroll
     for (int k = 0; k < 12; ++k) o[k] = cx((RO)(c * acc[k].re), (RO)(c * acc[k].im));
     Spin<SPO>::store(slot_wptr(S, slot_out, r, par), S.vh, s, o);
+  }
+  template <typename R, typename V>
+  __device__ __forceinline__ void write_rows(const SysDesc& S, int par, int r, int s, int row, Cx<R> (&a)[3],
+                                             Cx<R> (&b)[3], V&, bool ok) const {
+    if constexpr (COEF != C_ONE) {
+      const R c = coef<COEF, R>(S);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        a[k] = cx(c * a[k].re, c * a[k].im);
+        b[k] = cx(c * b[k].re, c * b[k].im);
+      }
+    }
+    store_rows<SPO>(slot_wptr(S, slot_out, r, par), S.vh, s, row, a, b, ok);
   }
 };
 
@@ -522,6 +548,28 @@ struct EpiXpay {
                                         typename RedT<R>::type& nrm) const {
     const Packed o = prepare(S, par, r, s, acc, nrm);
     commit(S, par, r, s, o);
+  }
+  template <typename R>
+  __device__ __forceinline__ void write_rows(const SysDesc& S, int par, int r, int s, int row, Cx<R> (&a)[3],
+                                             Cx<R> (&b)[3], typename RedT<R>::type& nrm, bool ok) const {
+    const char* xp = slot_ptr(S, slot_x, r, par);
+    const R c = coef<COEF, R>(S);
+    R n = (R)0;
+    Cx<R> x[3];
+    Spin<SPX>::load_spin(xp, S.vh, s, row, x);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      a[k] = cx(fma(c, a[k].re, x[k].re), fma(c, a[k].im, x[k].im));
+      if (RED) n = fma(a[k].re, a[k].re, fma(a[k].im, a[k].im, n));
+    }
+    Spin<SPX>::load_spin(xp, S.vh, s, 2 + row, x);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      b[k] = cx(fma(c, b[k].re, x[k].re), fma(c, b[k].im, x[k].im));
+      if (RED) n = fma(b[k].re, b[k].re, fma(b[k].im, b[k].im, n));
+    }
+    if (RED) nrm = to_red(n);
+    if (slot_out >= 0) store_rows<SPO>(slot_wptr(S, slot_out, r, par), S.vh, s, row, a, b, ok);
   }
 };
 
@@ -563,6 +611,20 @@ struct EpiXpayDot {
   }
 };
 
+// One spin of a residual, v <- bh - x + c v, and its |.|^2 added to n.
+template <int SPH, typename R>
+__device__ __forceinline__ void resid_spin(const char* xp, const char* bp, int vh, int s, int spin, R c, Cx<R> (&v)[3],
+                                           R& n) {
+  Cx<R> x[3], b[3];
+  Spin<SPH>::load_spin(xp, vh, s, spin, x);
+  Spin<SPH>::load_spin(bp, vh, s, spin, b);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    v[k] = cx(fma(c, v[k].re, b[k].re - x[k].re), fma(c, v[k].im, b[k].im - x[k].im));
+    n = fma(v[k].re, v[k].re, fma(v[k].im, v[k].im, n));
+  }
+}
+
 // Residual of the even-odd system in the high precision SPH at even site s,
 // once the accumulator x has absorbed the low-precision increment:
 //   r_hi = bh - x + kappa^2 * acc  (acc = H_eo t, t = H_oe x);  r_low <- r_hi;
@@ -592,6 +654,17 @@ struct EpiResidEO {
     Cx<typename Spin<SPL>::R> lo[12];
     convert12(rv, lo);
     Spin<SPL>::store(slot_wptr(S, S_R, r, par), S.vh, s, lo);
+  }
+  template <typename RH>
+  __device__ __forceinline__ void write_rows(const SysDesc& S, int par, int r, int s, int row, Cx<RH> (&a)[3],
+                                             Cx<RH> (&b)[3], typename RedT<RH>::type& nrm, bool ok) const {
+    const char *xp = slot_ptr(S, S_X, r, par), *bp = slot_ptr(S, S_BH, r, par);
+    const RH k2 = coef<C_PK2, RH>(S);
+    RH n = (RH)0;
+    resid_spin<SPH>(xp, bp, S.vh, s, row, k2, a, n);
+    resid_spin<SPH>(xp, bp, S.vh, s, 2 + row, k2, b, n);
+    nrm = to_red(n);
+    store_rows<SPL>(slot_wptr(S, S_R, r, par), S.vh, s, row, a, b, ok);
   }
 };
 
@@ -630,6 +703,18 @@ struct EpiResidFull {
       convert12(rv, lo);
       Spin<SPL>::store(slot_wptr(S, S_R, r, par), S.vh, s, lo);
     }
+  }
+  template <typename RH>
+  __device__ __forceinline__ void write_rows(const SysDesc& S, int par, int r, int s, int row, Cx<RH> (&a)[3],
+                                             Cx<RH> (&b)[3], typename RedT<RH>::type& nrm, bool ok) const {
+    const char *xp = slot_ptr(S, slot_x, r, par), *bp = slot_ptr(S, slot_b, r, par);
+    const RH kap = coef<C_PK, RH>(S);
+    RH n = (RH)0;
+    resid_spin<SPH>(xp, bp, S.vh, s, row, kap, a, n);
+    resid_spin<SPH>(xp, bp, S.vh, s, 2 + row, kap, b, n);
+    nrm = to_red(n);
+    if (slot_rt >= 0) store_rows<SPH>(slot_wptr(S, slot_rt, r, par), S.vh, s, row, a, b, ok);
+    if (STORE_LOW) store_rows<SPL>(slot_wptr(S, S_R, r, par), S.vh, s, row, a, b, ok);
   }
 };
 
@@ -850,34 +935,6 @@ __global__ void __launch_bounds__(256, HopOccupancy<SPA>::kMinBlocks)
         DW_HOP_DIR_W(1)
         DW_HOP_DIR_W(2)
         DW_HOP_DIR_W(3)
-      } else if constexpr (SPA == PDF) {
-        // compact loop: one copy of the double-float mat-vec per (U, U^dag)
-#pragma unroll 1
-        for (int mu = 0; mu < 4; ++mu) {
-          float eta;
-          Cx<R> h[6], g[6], u[9];
-          const DirSpin df = dir_spin(mu, SF), db = dir_spin(mu, SB);
-          const int nf = neighbour_rt(S, c, s, mu, +1, &eta);
-          project_rt_loaded(df, in, S, pin, r, nf, h);
-          Link<LP, C12>::load(ulink_own + mu * mu_stride, S.vh, s, u);
-          if (eta < 0.f) {
-#pragma unroll
-            for (int k = 0; k < 6; ++k) h[k] = cx(-h[k].re, -h[k].im);
-          }
-          su3_mul<false>(u, h, g);
-          accumulate_rt(df, acc, g);
-          const int nb = neighbour_rt(S, c, s, mu, -1, &eta);
-          project_rt_loaded(db, in, S, pin, r, nb, h);
-          Link<LP, C12>::load(ulink_nb + mu * mu_stride, S.vh, nb, u);
-          if (eta < 0.f) {
-#pragma unroll
-            for (int k = 0; k < 6; ++k) h[k] = cx(-h[k].re, -h[k].im);
-          }
-          su3_mul<true>(u, h, g);
-          accumulate_rt(db, acc, g);
-        }
-#pragma unroll
-        for (int k = 0; k < 12; ++k) acc[k] = cx(renorm(acc[k].re), renorm(acc[k].im));
       } else {
         DW_HOP_DIR(0)
         DW_HOP_DIR(1)
@@ -896,6 +953,217 @@ __global__ void __launch_bounds__(256, HopOccupancy<SPA>::kMinBlocks)
     } else if constexpr (Epi::kReduce) {
       DW_BLOCK_REDUCE(nrm)
     }
+  }
+}
+
+// ------------------------------------------------------------------ two threads per site
+// g = one row of the half spinor times U (or U^dag).
+template <bool ADJ>
+__device__ __forceinline__ void su3_mul_row(const Cx<double> (&u)[9], const Cx<double> (&h)[3], Cx<double> (&g)[3]) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (!ADJ) {
+      Cx<double> t = cmul(u[a * 3 + 0], h[0]);
+      t = cmadd(u[a * 3 + 1], h[1], t);
+      g[a] = cmadd(u[a * 3 + 2], h[2], t);
+    } else {
+      Cx<double> t = cjmul(u[0 * 3 + a], h[0]);
+      t = cjmadd(u[1 * 3 + a], h[1], t);
+      g[a] = cjmadd(u[2 * 3 + a], h[2], t);
+    }
+  }
+}
+// Double-float: the real and imaginary part of an output are the two lanes of
+// packed FP32x2 arithmetic.
+template <bool ADJ>
+__device__ __forceinline__ void su3_mul_row(const Cx<DF> (&u)[9], const Cx<DF> (&h)[3], Cx<DF> (&g)[3]) {
+  DF2 yr[3], yi[3];  // what the link's real and imaginary part multiply
+#pragma unroll
+  for (int b = 0; b < 3; ++b) {
+    yr[b].hi = make_float2(h[b].re.hi, h[b].im.hi);
+    yr[b].lo = make_float2(h[b].re.lo, h[b].im.lo);
+    yi[b].hi = ADJ ? make_float2(h[b].im.hi, -h[b].re.hi) : make_float2(-h[b].im.hi, h[b].re.hi);
+    yi[b].lo = ADJ ? make_float2(h[b].im.lo, -h[b].re.lo) : make_float2(-h[b].im.lo, h[b].re.lo);
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    DF x[6];
+    DF2 y[6];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const Cx<DF> m = ADJ ? u[b * 3 + a] : u[a * 3 + b];
+      x[2 * b] = m.re;
+      y[2 * b] = yr[b];
+      x[2 * b + 1] = m.im;
+      y[2 * b + 1] = yi[b];
+    }
+    const DF2 t = df2_dot6(x, y);
+    g[a] = cx(df_make(t.hi.x, t.lo.x), df_make(t.hi.y, t.lo.y));
+  }
+}
+// sign flips by mask (0 or the sign bit): bit operations, so that IEEE FP64
+// negations stay off the FP64 pipe
+__device__ __forceinline__ double flip(double v, uint32_t m) {
+  return __hiloint2double(__double2hiint(v) ^ (int)m, __double2loint(v));
+}
+__device__ __forceinline__ float flip(float v, uint32_t m) { return __uint_as_float(__float_as_uint(v) ^ m); }
+__device__ __forceinline__ DF flip(DF v, uint32_t m) { return df_make(flip(v.hi, m), flip(v.lo, m)); }
+// +-1 (or +-i) times q, the sign by mask
+template <bool IMAG, typename R>
+__device__ __forceinline__ Cx<R> times_unit(Cx<R> q, uint32_t m) {
+  return IMAG ? cx(flip(q.im, m ^ 0x80000000u), flip(q.re, m)) : cx(flip(q.re, m), flip(q.im, m));
+}
+__device__ __forceinline__ Cx<double> row_add(Cx<double> a, Cx<double> b) { return a + b; }
+__device__ __forceinline__ Cx<DF> row_add(Cx<DF> a, Cx<DF> b) { return cadd_lazy(a, b); }
+
+// One row of the half spinor projected from neighbour n: h = p_row + c p_q,
+// c = +-1 or +-i with the sign by mask cm; bm flips h on the t-boundary slice.
+template <int SPA, bool IMAG, typename R>
+__device__ __forceinline__ void row_project(const char* in, int vh, int n, int row, int partner, uint32_t cm,
+                                            uint32_t bm, Cx<R> (&h)[3]) {
+  Cx<R> q[3];
+  Spin<SPA>::load_spin(in, vh, n, row, h);
+  Spin<SPA>::load_spin(in, vh, n, partner, q);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    h[c] = row_add(h[c], times_unit<IMAG>(q[c], cm));
+    h[c] = cx(flip(h[c].re, bm), flip(h[c].im, bm));
+  }
+}
+
+// Both directions of one mu for one row.  With g_f = U h_f and g_b = U^dag h_b
+// the upper spin takes g_f + g_b and the lower spin d (g_f - g_b), d the unit
+// factor of the forward projector (the backward one is its negative).
+template <int SPA, bool C12, bool IMAG, typename R>
+__device__ __forceinline__ void row_mu(const SysDesc& S, const char* in, const char* own, const char* nbr, int s, int nf,
+                                       int nb, int row, int partner, uint32_t cm, uint32_t dm, uint32_t bf, uint32_t bb,
+                                       Cx<R> (&up)[3], Cx<R> (&low)[3], bool first_up, bool first_low) {
+  Cx<R> h[3], g[3], u[9];
+  row_project<SPA, IMAG>(in, S.vh, nf, row, partner, cm, bf, h);
+  Link<SPA, C12>::load(own, S.vh, s, u);
+  su3_mul_row<false>(u, h, g);
+  row_project<SPA, IMAG>(in, S.vh, nb, row, partner, cm ^ 0x80000000u, bb, h);
+  Link<SPA, C12>::load(nbr, S.vh, nb, u);
+  if constexpr (SPA == P64) {
+    // The FP64 pipe (64 cycles per warp instruction) is the bound, so additions
+    // are saved: the backward product's chain starts from g_f and yields
+    // A = g_f + g_b at no extra cost, and g_f - g_b = 2 g_f - A is one FMA:
+    // 18 instead of 24 operations per mu and row, none onto empty sums.
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      Cx<R> t = cjmadd(u[0 * 3 + a], h[0], g[a]);
+      t = cjmadd(u[1 * 3 + a], h[1], t);
+      t = cjmadd(u[2 * 3 + a], h[2], t);
+      const Cx<R> d = times_unit<IMAG>(cx(fma(2.0, g[a].re, -t.re), fma(2.0, g[a].im, -t.im)), dm);
+      up[a] = first_up ? t : up[a] + t;
+      low[a] = first_low ? d : low[a] + d;
+    }
+  } else {
+    Cx<R> gb[3];
+    su3_mul_row<true>(u, h, gb);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      up[a] = row_add(row_add(up[a], g[a]), gb[a]);
+      low[a] = row_add(low[a], times_unit<IMAG>(g[a], dm));
+      low[a] = row_add(low[a], times_unit<IMAG>(gb[a], dm ^ 0x80000000u));
+    }
+  }
+}
+
+// The FP64-class Wilson stencils (IEEE FP64 and double-float): two threads per
+// output site, one per row of the half spinor; lanes 0-15 of a warp take row 0
+// and lanes 16-31 row 1 of 16 consecutive sites, so that one load instruction
+// serves both rows' links.  Row 0 pairs with spin 3 and row 1 with spin 2 for
+// mu = x, y, with 2 and 3 for z, t.  A thread holds its upper spin and one
+// lower spin: through x and y it collects the other row's lower spin, then the
+// rows swap what they collected and go on with their own through z and t.
+// Unit factors of (1 + s gamma_mu), h = p_row + c p_partner, lower = d g:
+//   x: c = -s i, d = s i (both rows)   y: c = d = -s (row 0), s (row 1)
+//   t: c = s, d = s (both rows)        z: c = -s i, d = s i (row 0), the opposite (row 1)
+// Blocks: T sites x RB right-hand sides, 2 T RB threads.
+#ifndef DW_ROWS_ATTR
+#define DW_ROWS_ATTR __launch_bounds__(512, 1)
+#endif
+template <int SPA, bool C12, bool DAG, class Epi>
+__global__ void DW_ROWS_ATTR
+    k_hop_rows(const __grid_constant__ Batch B, int par_mode, int link_slot, int in_slot, Epi epi, RedArgs ra) {
+  static_assert(SPA == P64 || SPA == PDF, "two threads per site: FP64-class storage");
+  using R = typename Spin<SPA>::R;
+  const int T = B.T, RB = B.RB;
+  const unsigned bx = B.rev ? gridDim.x - 1u - blockIdx.x : blockIdx.x;
+  int by = 0, b = (int)bx, par, rl = 0;
+  if (B.ny > 1) {
+    b = (int)(bx / (unsigned)B.ny);
+    by = (int)bx - b * B.ny;
+  }
+  if (par_mode == 2) {
+    par = b >= B.ntot ? 1 : 0;
+    b -= par * B.ntot;
+  } else {
+    par = par_mode;
+  }
+  const SysDesc& S = B.sd[block_system(B, b)];
+  if (RB > 1) rl = (int)threadIdx.x / (2 * T);
+  const int r = by * RB + rl;
+  const int tile = b - S.tile0;
+  const int row = (threadIdx.x >> 4) & 1;
+  const int at = ((((int)threadIdx.x - rl * 2 * T) >> 5) << 4) + (threadIdx.x & 15);
+  const int s0 = tile * T + at;
+  const bool ok = s0 < S.vh;
+  // a warp works on one right-hand side: the gate is the same for all its
+  // lanes, and lanes past the last site repeat site 0 without storing
+  typename RedT<R>::type nrm = red_zero(typename RedT<R>::type());
+  if (r < S.nrhs && gate_of(epi.gate, ra.cols, S.col0 + r)) {
+    const int s = ok ? s0 : 0;
+    const Coord c = coord_of(S, s, par);
+    const int pin = par ^ 1;
+    const char* in = slot_ptr(S, in_slot, r, pin);
+    const char* own = slot_ptr(S, link_slot, 0, par);
+    const char* nbr = slot_ptr(S, link_slot, 0, pin);
+    const long long mu_stride = (long long)Link<SPA, C12>::kBytes * S.vh;
+    constexpr uint32_t kS = DAG ? 0u : 0x80000000u;  // sign of the forward projector's s
+    const uint32_t row1 = row ? 0x80000000u : 0u;
+    Cx<R> up[3], low[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) up[k] = low[k] = cx((R)0, (R)0);
+    // x and y, then z and t: one copy of the code for both halves, which keeps
+    // the kernel inside the instruction cache
+#pragma unroll 1
+    for (int ph = 0; ph < 2; ++ph) {
+      const int partner = ph == 0 ? 3 - row : 2 + row;
+      float ef, eb;
+      int nf = ph == 0 ? neighbour<0, +1>(S, c, s, &ef) : neighbour<2, +1>(S, c, s, &ef);
+      int nb = ph == 0 ? neighbour<0, -1>(S, c, s, &eb) : neighbour<2, -1>(S, c, s, &eb);
+      const uint32_t mi = kS ^ (ph == 0 ? 0u : row1);
+      row_mu<SPA, C12, true>(S, in, own, nbr, s, nf, nb, row, partner, mi ^ 0x80000000u, mi, 0u, 0u, up, low, ph == 0,
+                             ph == 0);
+      own += mu_stride;
+      nbr += mu_stride;
+      nf = ph == 0 ? neighbour<1, +1>(S, c, s, &ef) : neighbour<3, +1>(S, c, s, &ef);
+      nb = ph == 0 ? neighbour<1, -1>(S, c, s, &eb) : neighbour<3, -1>(S, c, s, &eb);
+      const uint32_t mr = kS ^ (ph == 0 ? row1 ^ 0x80000000u : 0u);
+      row_mu<SPA, C12, false>(S, in, own, nbr, s, nf, nb, row, partner, mr, mr, __float_as_uint(ef) & 0x80000000u,
+                              __float_as_uint(eb) & 0x80000000u, up, low, false, false);
+      own += mu_stride;
+      nbr += mu_stride;
+      if (ph == 0) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) low[k] = other_row(low[k]);
+      }
+    }
+    if constexpr (SPA == PDF) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        up[k] = cx(renorm(up[k].re), renorm(up[k].im));
+        low[k] = cx(renorm(low[k].re), renorm(low[k].im));
+      }
+    }
+    epi.write_rows(S, par, r, s, row, up, low, nrm, ok);
+    if (!ok) nrm = red_zero(typename RedT<R>::type());
+  }
+  if constexpr (Epi::kReduce) {
+    const int ntiles = par_mode == 2 ? 2 * S.tpp : S.tpp;
+    reduce_block(S, 2 * T, RB, par_mode == 2 ? par * S.tpp + tile : tile, ntiles, nrm, ra, by);
   }
 }
 
