@@ -419,7 +419,7 @@ dw_status derived_links(dw_field* U, int prec, int c12, cudaStream_t st, const c
   d.prec = prec;
   d.c12 = c12;
   d.bytes = 8ull * link_bytes(prec, c12) * vh_of(U->lat);
-  DW_CUDA(cudaMalloc(&d.ptr, d.bytes));
+  DW_CUDA(device_alloc(&d.ptr, d.bytes));
   d.version = U->version - 1;  // force conversion below
   U->derived.push_back(d);
   return derived_links(U, prec, c12, st, out);
@@ -463,15 +463,25 @@ static void tune_load_once() {
   }
   fclose(f);
 }
-std::string tune_key(const dw_lattice* lats, int n, int nrhs, int prec, int c12) {
-  char dev_name[256] = "gpu";
+// A device's name, asked for once: cudaGetDeviceProperties costs microseconds
+// and every operator application looks its block shape up.
+static std::string device_name() {
+  static std::mutex mu;
+  static std::map<int, std::string> names;
   int dev = 0;
-  cudaDeviceProp prop;
-  if (cudaGetDevice(&dev) == cudaSuccess && cudaGetDeviceProperties(&prop, dev) == cudaSuccess)
-    snprintf(dev_name, sizeof dev_name, "%s", prop.name);
-  for (char* c = dev_name; *c; ++c)
-    if (*c == ' ') *c = '_';
-  std::string key = std::string(dev_name) + "/v5/" + prec_name(prec) + (c12 ? "c12" : "c18") + "/r" +
+  if (cudaGetDevice(&dev) != cudaSuccess) return "gpu";
+  std::lock_guard<std::mutex> lock(mu);
+  std::string& name = names[dev];
+  if (name.empty()) {
+    cudaDeviceProp prop;
+    name = cudaGetDeviceProperties(&prop, dev) == cudaSuccess ? prop.name : "gpu";
+    for (char& c : name)
+      if (c == ' ') c = '_';
+  }
+  return name;
+}
+std::string tune_key(const dw_lattice* lats, int n, int nrhs, int prec, int c12) {
+  std::string key = device_name() + "/v6/" + prec_name(prec) + (c12 ? "c12" : "c18") + "/r" +
                     std::to_string(nrhs);
   for (int i = 0; i < n; ++i)
     key += "/" + std::to_string(lats[i].dims[0]) + "x" + std::to_string(lats[i].dims[1]) + "x" +
@@ -618,7 +628,7 @@ static dw_status make_field(const dw_lattice* lat, dw_kind kind, dw_prec prec, i
   f->version = 1;
   cudaGetDevice(&f->device);
   if (owned) {
-    cudaError_t e = cudaMalloc(&f->ptr, need);
+    cudaError_t e = device_alloc(&f->ptr, need);
     if (e != cudaSuccess) {
       delete f;
       return cuda_error(e, "cudaMalloc(field)", __FILE__, __LINE__);
@@ -686,7 +696,7 @@ dw_status dw_field_export(const dw_field* f, double* dev, dw_stream_t stream) {
   return unpack_range(f, dev, 0, canonical_units(f), reinterpret_cast<cudaStream_t>(stream));
 }
 
-// Staging buffers for host transfers come from a stream-ordered memory pool
+// Staging buffers for host transfers and the operators' temporaries come from a stream-ordered memory pool
 // owned by the library (one per device), which keeps up to kStagingKeep bytes
 // reserved between calls so that repeated transfers do not reallocate.
 static constexpr uint64_t kStagingKeep = 8ull << 30;
@@ -713,6 +723,31 @@ static dw_status staging_pool(cudaMemPool_t* out) {
   *out = g_pool[dev];
   return DW_OK;
 }
+
+}  // extern "C"
+dw_status dw::scratch_alloc(char** p, size_t nb, cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    DW_CUDA(cudaMallocAsync(reinterpret_cast<void**>(p), nb, st));  // an allocation node of the caller's graph
+    return DW_OK;
+  }
+  cudaMemPool_t pool;
+  DW_TRY(staging_pool(&pool));
+  DW_CUDA(cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), nb, pool, st));
+  return DW_OK;
+}
+cudaError_t dw::device_alloc(char** p, size_t nb) {
+  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), nb);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaMemPool_t pool;
+    (void)cudaGetLastError();
+    if (staging_pool(&pool) == DW_OK && cudaDeviceSynchronize() == cudaSuccess &&
+        cudaMemPoolTrimTo(pool, 0) == cudaSuccess)
+      e = cudaMalloc(reinterpret_cast<void**>(p), nb);
+  }
+  return e;
+}
+extern "C" {
 
 // Large host transfers run in chunks: the DMA copies go on a copy stream owned
 // by the library (one per device) and the layout kernels on the caller's
@@ -768,10 +803,8 @@ dw_status dw_field_upload(dw_field* f, const double* host, dw_stream_t stream) {
   const long long nu = canonical_units(f);
   const size_t ub = canonical_unit_bytes(f);
   const size_t nb = (size_t)nu * ub;
-  cudaMemPool_t pool;
-  DW_TRY(staging_pool(&pool));
   char* tmp = nullptr;
-  DW_CUDA(cudaMallocFromPoolAsync(reinterpret_cast<void**>(&tmp), nb, pool, st));
+  DW_TRY(scratch_alloc(&tmp, nb, st));
   const char* h = reinterpret_cast<const char*>(host);
   f->version += 1;
   const int n = transfer_chunks(nb, st);
@@ -815,10 +848,8 @@ dw_status dw_field_download(const dw_field* f, double* host, dw_stream_t stream)
   const long long nu = canonical_units(f);
   const size_t ub = canonical_unit_bytes(f);
   const size_t nb = (size_t)nu * ub;
-  cudaMemPool_t pool;
-  DW_TRY(staging_pool(&pool));
   char* tmp = nullptr;
-  DW_CUDA(cudaMallocFromPoolAsync(reinterpret_cast<void**>(&tmp), nb, pool, st));
+  DW_TRY(scratch_alloc(&tmp, nb, st));
   char* h = reinterpret_cast<char*>(host);
   const int n = transfer_chunks(nb, st);
   dw_status s = DW_OK;

@@ -126,7 +126,7 @@ static dw_status temp_like(const dw_field* f, cudaStream_t st, dw_field* t) {
   t->bytes = f->bytes;
   t->owned = 0;
   t->version = 1;
-  DW_CUDA(cudaMallocAsync((void**)&t->ptr, f->bytes, st));
+  DW_TRY(scratch_alloc(&t->ptr, f->bytes, st));
   return DW_OK;
 }
 

@@ -101,6 +101,14 @@ void tune_store(const std::string& key, BlockShape v);
 // Key of the tuning cache: device name, storage, nrhs and every lattice.
 std::string tune_key(const dw_lattice* lats, int n, int nrhs, int prec, int c12);
 
+// Stream-ordered device scratch from the library's pool (freed with
+// cudaFreeAsync), which keeps released memory between calls: from the default
+// pool, whose memory goes back to the driver at every synchronisation, the
+// first call after one paid about 200 us for mapping it again.
+dw_status scratch_alloc(char** p, size_t nb, cudaStream_t st);
+// cudaMalloc; when memory is short, what that pool keeps is given back first.
+cudaError_t device_alloc(char** p, size_t nb);
+
 // Device scratch for reductions of one plan.
 struct RedBuf {
   DF* partial = nullptr;

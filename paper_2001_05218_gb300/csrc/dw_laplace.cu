@@ -47,7 +47,7 @@ extern "C" dw_status dw_laplace_apply(const dw_field* U, const dw_field* in, dw_
   char* tmp = nullptr;
   if (in->kind != DW_SPINOR_FULL) {
     const size_t nb = (size_t)in->nrhs * spin_bytes(in->prec) * vh_of(in->lat);
-    DW_CUDA(cudaMallocAsync((void**)&tmp, nb, st));
+    DW_TRY(scratch_alloc(&tmp, nb, st));
     S.f[S_AUX1] = arena_slot(tmp, in->lat, in->prec, in->nrhs, 1);
   }
   const bool c12 = U->compress12 != 0;

@@ -34,7 +34,7 @@ static dw_status apply_one(const dw_field* U, const dw_field* in, dw_field* out,
   char* tmp = nullptr;
   if (in->kind != DW_SPINOR_FULL) {
     const size_t nb = (size_t)in->nrhs * spin_bytes(in->prec) * vh_of(in->lat);
-    DW_CUDA(cudaMallocAsync((void**)&tmp, nb, st));
+    DW_TRY(scratch_alloc(&tmp, nb, st));
     S.f[S_AUX1] = arena_slot(tmp, in->lat, in->prec, in->nrhs, 1);
   }
   dw_status s = apply_dispatch<false>(E, U, in, dag);
@@ -64,7 +64,7 @@ dw_status dw_normal_apply(const dw_field* U, const dw_field* in, dw_field* out, 
   dw_field mid = *out;  // same shape as out, memory from the stream-ordered pool
   mid.derived.clear();
   mid.owned = 0;
-  DW_CUDA(cudaMallocAsync((void**)&mid.ptr, out->bytes, st));
+  DW_TRY(scratch_alloc(&mid.ptr, out->bytes, st));
   dw_status s = apply_one(U, in, &mid, 0, st);
   if (s == DW_OK) s = apply_one(U, &mid, out, 1, st);
   cudaFreeAsync(mid.ptr, st);

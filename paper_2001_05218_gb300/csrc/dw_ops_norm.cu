@@ -26,7 +26,7 @@ extern "C" dw_status dw_apply_norm(const dw_field* U, const dw_field* in, dw_fie
   const size_t part_b = al(sizeof(DF) * E.P.partials);
   const size_t cols_b = al(sizeof(ColState) * E.P.ncols), flags_b = al(sizeof(Flags));
   char* buf = nullptr;
-  DW_CUDA(cudaMallocAsync((void**)&buf, tmp_b + part_b + cols_b + flags_b, st));
+  DW_TRY(scratch_alloc(&buf, tmp_b + part_b + cols_b + flags_b, st));
   char* p = buf;
   if (tmp_b) S.f[S_AUX1] = arena_slot(p, in->lat, in->prec, in->nrhs, 1);
   p += tmp_b;

@@ -337,7 +337,7 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
       }
     }
     const size_t red_bytes = al(sizeof(DF) * F.P.partials) + al(sizeof(ColState) * F.P.ncols) + al(sizeof(Flags));
-    DW_CUDA(cudaMalloc((void**)&fresh.arena, total + red_bytes));
+    DW_CUDA(device_alloc(&fresh.arena, total + red_bytes));
     char* rp = fresh.arena + total;
     F.rb.partial = reinterpret_cast<DF*>(rp);
     rp += al(sizeof(DF) * F.P.partials);
