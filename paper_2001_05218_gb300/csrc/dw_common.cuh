@@ -916,7 +916,7 @@ struct alignas(16) ColState {
   int xzero;       // initial guess is zero: the first residual is the source itself
   int restart;     // defect correction: the next beta is 0 (new search direction)
   int zsrc;        // zero source: the solution is x = 0
-  int pad;
+  int zr;          // 1: z = r (plain CG), so |z|^2 is the |r|^2 just formed
 };
 
 // Batch-wide flags.
@@ -965,7 +965,19 @@ __device__ __forceinline__ void deactivate(ColState& C, Flags* F, int status) {
   }
 }
 
-// CG scalar recurrences on one column's state, run by one thread.
+// beta = |z|^2 / |z_old|^2 (0 at a restart); gamma = |z|^2
+__device__ __forceinline__ void form_beta(ColState& C, double v) {
+  C.beta = C.restart ? 0.0 : v / C.gamma;
+  C.beta_f = (float)C.beta;
+  C.restart = 0;
+  C.gamma = v;
+}
+
+// CG scalar recurrences on one column's state, run by one thread.  Where z = r
+// (zr) the update of r, or the reliable update that replaces r, also forms
+// beta: |z|^2 is the sum at hand, and neither a pass over r nor a second
+// reduction is needed for it (k_norm and its finishing kernel took 9.6 of 93 us
+// per iteration on the 16^3x32 normal equations in FP32).
 __device__ __forceinline__ void finalize(const RedArgs& ra, ColState& C, double v) {
   switch (ra.fin) {
     case FIN_STORE0: C.store[0] = v; break;
@@ -1002,6 +1014,8 @@ __device__ __forceinline__ void finalize(const RedArgs& ra, ColState& C, double 
       } else if (v <= C.tol2 || v < C.delta2 * C.rr_ref || C.iter >= C.maxiter || timeout) {
         C.do_rel = 1;
         atomicAdd(&ra.flags->rel_pending, 1);
+      } else if (C.zr) {
+        form_beta(C, v);
       }
       break;
     }
@@ -1035,6 +1049,7 @@ __device__ __forceinline__ void finalize(const RedArgs& ra, ColState& C, double 
       else if (!isfinite(v)) deactivate(C, ra.flags, 7);
       else if (C.iter >= C.maxiter) deactivate(C, ra.flags, 6 /* NOT_CONVERGED */);
       else if (timeout) deactivate(C, ra.flags, 8 /* TIMEOUT */);
+      if (C.active && C.zr) form_beta(C, v);
       break;
     }
     case FIN_GAMMA0:
@@ -1045,10 +1060,7 @@ __device__ __forceinline__ void finalize(const RedArgs& ra, ColState& C, double 
       break;
     case FIN_BETA:
       if (!C.active) break;
-      C.beta = C.restart ? 0.0 : v / C.gamma;
-      C.beta_f = (float)C.beta;
-      C.restart = 0;
-      C.gamma = v;
+      form_beta(C, v);
       break;
   }
 }

@@ -41,6 +41,8 @@ namespace dw {
 enum Mode { MODE_EO = 0, MODE_FULL = 1, MODE_NORMAL = 2, MODE_HERM = 3 };
 // modes whose CG vectors live on the even sites only
 inline bool eo_mode(int mode) { return mode == MODE_EO || mode == MODE_HERM; }
+// plain CG: the search direction is built from r itself
+inline bool z_is_r(int mode) { return mode == MODE_NORMAL || mode == MODE_HERM; }
 
 struct SolveArgs {
   int n;
@@ -99,8 +101,11 @@ struct CG {
     }
   }
 
-  // z = A-side residual and its norm with finalizer fin (FIN_GAMMA0 / FIN_BETA)
+  // z = A-side residual and its norm with finalizer fin (FIN_GAMMA0 / FIN_BETA);
+  // where z aliases r, |z|^2 is only summed for the first iteration: after
+  // that FIN_UPDATE and FIN_RELIABLE form beta from the |r|^2 they have
   static void zstep(const Exec& E, int mode, int fin) {
+    if (z_is_r(mode) && fin == FIN_BETA) return;
     if constexpr (OP == OP_LAPLACE) {
       norm<L>(E, 0, S_R, fin);  // MODE_HERM: z aliases r
     } else if (mode == MODE_EO) {
@@ -355,7 +360,7 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
       S.f[S_X] = S.f[S_XU];
       for (size_t k = 0; k < pieces.size(); ++k)
         S.f[pieces[k].slot] = arena_slot(fresh.arena + poff[i][k], lats[i], pieces[k].prec, nrhs, pieces[k].npar);
-      if (mode == MODE_NORMAL || mode == MODE_HERM) S.f[S_Z] = S.f[S_R];
+      if (z_is_r(mode)) S.f[S_Z] = S.f[S_R];
       for (auto pc : {S_XL, S_P})
         fresh.zero.push_back({S.f[pc].p, (size_t)nrhs * fpar * (pc == S_XL ? spin_bytes(A) : spin_bytes(L)) * S.vh});
       // odd half of the high-precision temporary: holds H_oe x_e after every
@@ -385,6 +390,7 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
     c.delta2 = (L == P64 || L == PDF) ? 0.0 : a.p.delta * a.p.delta;
     c.maxiter = a.p.maxiter;
     c.defect = a.p.defect_correction ? 1 : 0;
+    c.zr = z_is_r(mode) ? 1 : 0;
     c.active = 1;
     c.do_rel = 1;  // the first FP64 residual is a "reliable update" unless x0 = 0
     c.status = DW_ERR_NOT_CONVERGED;
