@@ -852,20 +852,31 @@ __device__ __forceinline__ void laplace_dirs(const SysDesc& S, const In& in, con
 // par_mode 0/1: output parity fixed, grid = ntot blocks.  par_mode 2: both
 // parities, grid = 2*ntot (block b >= ntot works on odd output sites).
 // Input is read on the opposite parity.  SPA: arithmetic-precision tag.
-// Minimum resident blocks (of 256 threads) per SM requested from the compiler.
-// Measured on GB300: capping the double-float stencil at 128 registers (2)
-// runs 9% faster despite small spills (more warps to hide its long dependency
-// chains); the 16-bit stencils, whose operands stay in packed 16-bit words,
-// fit 80 registers without spills (3) and run 5% faster there than at 128.
+// Minimum resident blocks (of 256 threads) per SM requested from the compiler,
+// that is a register cap (256 threads x n blocks share 65536 registers).  The
+// kernels are bound by load latency at the occupancy that this leaves.
+// Measured on GB300, microseconds per even-site application at 32^3x64:
+//   FP16, 12 reals   2: 145.6   3: 142.5   4: 138.0 (with |out|^2 193 -> 184)
+//   FP32, 18 reals   1: 284.5   2: 252.9   3: 306 (spills)
+//   FP32, 12 reals   1: 224.0   2: 211.2   3: 224
+//   I16, 12 reals    1: 181.8   2: 182.0   3: 179.4
+// Double-float (the Laplacian; the Wilson form has its own kernel): 2.
 #ifndef DW_HOP16_MINB
-#define DW_HOP16_MINB 3
+#define DW_HOP16_MINB 4
 #endif
-#ifndef DW_HOPDF_MINB
-#define DW_HOPDF_MINB 2
+#ifndef DW_HOP32_MINB
+#define DW_HOP32_MINB 2
+#endif
+#ifndef DW_HOPI16_MINB
+#define DW_HOPI16_MINB 3
 #endif
 template <int SPA>
 struct HopOccupancy {
-  static constexpr int kMinBlocks = (SPA == P16 || SPA == PB16) ? DW_HOP16_MINB : SPA == PDF ? DW_HOPDF_MINB : 1;
+  static constexpr int kMinBlocks = (SPA == P16 || SPA == PB16) ? DW_HOP16_MINB
+                                    : SPA == PDF                ? 2
+                                    : SPA == P32                ? DW_HOP32_MINB
+                                    : SPA == PI16               ? DW_HOPI16_MINB
+                                                                : 1;
 };
 
 template <int SPA, int LP, bool C12, bool DAG, class In, class Epi, int OP = OP_WILSON>
