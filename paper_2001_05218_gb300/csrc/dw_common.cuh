@@ -381,6 +381,12 @@ DW_HW_SPECIALISE(PB16, "bf16", 0x3F80BF80u, 0xBF803F80u)
 #undef DW_HW_SPECIALISE
 
 // ------------------------------------------------------------------ spinor storage
+// Spinors are read with plain (coherent) loads: the one-kernel loop reads what
+// other blocks of the same launch wrote before its grid barrier, which the
+// read-only path does not promise to see.
+template <typename T>
+__device__ __forceinline__ T ld_field(const T* p) { return *p; }
+
 template <int P>
 struct Spin;
 
@@ -393,7 +399,7 @@ struct Spin<P64> {
     const double2* b = reinterpret_cast<const double2*>(base);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      double2 t = __ldg(b + (size_t)k * vh + s);
+      double2 t = ld_field(b + (size_t)k * vh + s);
       v[k] = cx(t.x, t.y);
     }
   }
@@ -422,7 +428,7 @@ struct Spin<P64> {
     const double2* b = reinterpret_cast<const double2*>(base) + (size_t)(3 * spin) * vh + s;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      double2 t = __ldg(b + (size_t)c * vh);
+      double2 t = ld_field(b + (size_t)c * vh);
       v[c] = cx(t.x, t.y);
     }
   }
@@ -442,7 +448,7 @@ struct Spin<P32> {
     const float4* b = reinterpret_cast<const float4*>(base);
 #pragma unroll
     for (int k = 0; k < 6; ++k) {
-      float4 t = __ldg(b + (size_t)k * vh + s);
+      float4 t = ld_field(b + (size_t)k * vh + s);
       v[2 * k] = cx(t.x, t.y);
       v[2 * k + 1] = cx(t.z, t.w);
     }
@@ -465,6 +471,21 @@ struct Spin<P32> {
     store_packed(base, vh, s, pack(v));
   }
   __device__ static __forceinline__ void roundtrip(Cx<float> (&)[12]) {}
+  // load in two steps: the words, and their values
+  __device__ static __forceinline__ Packed load_packed(const char* base, int vh, int s) {
+    const float4* b = reinterpret_cast<const float4*>(base);
+    Packed o;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) o.w[k] = ld_field(b + (size_t)k * vh + s);
+    return o;
+  }
+  __device__ static __forceinline__ void unpack(const Packed& o, Cx<float> (&v)[12]) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      v[2 * k] = cx(o.w[k].x, o.w[k].y);
+      v[2 * k + 1] = cx(o.w[k].z, o.w[k].w);
+    }
+  }
 };
 
 // Largest component magnitude of a site, the per-site scale of 16-bit
@@ -488,10 +509,10 @@ struct Spin16 {
   // value = v * sc
   __device__ static __forceinline__ void load_raw(const char* base, int vh, int s, Cx<float> (&v)[12], float& sc) {
     const uint4* b = reinterpret_cast<const uint4*>(base);
-    sc = __ldg(reinterpret_cast<const float*>(base + (size_t)48 * vh) + s) * (1.f / H16<P>::kUnit);
+    sc = ld_field(reinterpret_cast<const float*>(base + (size_t)48 * vh) + s) * (1.f / H16<P>::kUnit);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      uint4 t = __ldg(b + (size_t)k * vh + s);
+      uint4 t = ld_field(b + (size_t)k * vh + s);
       float2 a = H16<P>::to2(t.x), c = H16<P>::to2(t.y), d = H16<P>::to2(t.z), e = H16<P>::to2(t.w);
       v[4 * k + 0] = cx(a.x, a.y);
       v[4 * k + 1] = cx(c.x, c.y);
@@ -502,10 +523,10 @@ struct Spin16 {
   // stored words (one complex per word, see HW) and the site's scale
   __device__ static __forceinline__ void load_words(const char* base, int vh, int s, uint32_t (&w)[12], float& sc) {
     const uint4* b = reinterpret_cast<const uint4*>(base);
-    sc = __ldg(reinterpret_cast<const float*>(base + (size_t)48 * vh) + s);
+    sc = ld_field(reinterpret_cast<const float*>(base + (size_t)48 * vh) + s);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      const uint4 t = __ldg(b + (size_t)k * vh + s);
+      const uint4 t = ld_field(b + (size_t)k * vh + s);
       w[4 * k + 0] = t.x;
       w[4 * k + 1] = t.y;
       w[4 * k + 2] = t.z;
@@ -514,10 +535,10 @@ struct Spin16 {
   }
   __device__ static __forceinline__ void load(const char* base, int vh, int s, Cx<float> (&v)[12]) {
     const uint4* b = reinterpret_cast<const uint4*>(base);
-    const float sc = __ldg(reinterpret_cast<const float*>(base + (size_t)48 * vh) + s) * (1.f / H16<P>::kUnit);
+    const float sc = ld_field(reinterpret_cast<const float*>(base + (size_t)48 * vh) + s) * (1.f / H16<P>::kUnit);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      uint4 t = __ldg(b + (size_t)k * vh + s);
+      uint4 t = ld_field(b + (size_t)k * vh + s);
       float2 a = H16<P>::to2(t.x), c = H16<P>::to2(t.y), d = H16<P>::to2(t.z), e = H16<P>::to2(t.w);
       v[4 * k + 0] = cx(a.x * sc, a.y * sc);
       v[4 * k + 1] = cx(c.x * sc, c.y * sc);
@@ -551,6 +572,27 @@ struct Spin16 {
   __device__ static __forceinline__ void store(char* base, int vh, int s, const Cx<float> (&v)[12]) {
     store_packed(base, vh, s, pack(v));
   }
+  // load in two steps: the words, and their values
+  __device__ static __forceinline__ Packed load_packed(const char* base, int vh, int s) {
+    const uint4* b = reinterpret_cast<const uint4*>(base);
+    Packed o;
+    o.m = ld_field(reinterpret_cast<const float*>(base + (size_t)48 * vh) + s);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) o.w[k] = ld_field(b + (size_t)k * vh + s);
+    return o;
+  }
+  __device__ static __forceinline__ void unpack(const Packed& o, Cx<float> (&v)[12]) {
+    const float sc = o.m * (1.f / H16<P>::kUnit);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const uint32_t w[4] = {o.w[k].x, o.w[k].y, o.w[k].z, o.w[k].w};
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float2 a = H16<P>::to2(w[j]);
+        v[4 * k + j] = cx(a.x * sc, a.y * sc);
+      }
+    }
+  }
   __device__ static __forceinline__ void roundtrip(Cx<float> (&v)[12]) {
     const float m = site_max(v);
     const float inv = m > 0.f ? 1.0f / m : 0.f;
@@ -579,7 +621,7 @@ struct Spin<PDF> {
     const float4* b = reinterpret_cast<const float4*>(base);
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-      float4 t = __ldg(b + (size_t)k * vh + s);
+      float4 t = ld_field(b + (size_t)k * vh + s);
       v[k].re = df_make(t.x, t.y);
       v[k].im = df_make(t.z, t.w);
     }
@@ -606,7 +648,7 @@ struct Spin<PDF> {
     const float4* b = reinterpret_cast<const float4*>(base) + (size_t)(3 * spin) * vh + s;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      float4 t = __ldg(b + (size_t)c * vh);
+      float4 t = ld_field(b + (size_t)c * vh);
       v[c].re = df_make(t.x, t.y);
       v[c].im = df_make(t.z, t.w);
     }
@@ -927,6 +969,11 @@ struct Flags {
   int max_loops;    // hard cap on loops (maxiter + 2)
   int rel_runs;     // reliable-update passes run by the device-driven loop
   int fin_count;    // columns that the running k_finish has finished (0 between launches)
+  // grid barrier of the one-kernel loop (k_cg_loop): arrivals of this solve, and
+  // their number at the end of the last launch
+  unsigned bar_count, bar_base;
+  int bar_error;    // 1: a barrier gave up waiting
+  int late;         // 1: the deadline has passed (decided by one block for all)
 };
 
 enum Fin {
@@ -973,6 +1020,27 @@ __device__ __forceinline__ void form_beta(ColState& C, double v) {
   C.gamma = v;
 }
 
+// alpha = gamma / v; false: p^dag A p <= 0 or not finite, CG cannot continue
+__device__ __forceinline__ bool form_alpha(ColState& C, double v) {
+  if (!(v > 0.0) || !isfinite(v) || !isfinite(C.gamma)) return false;
+  C.alpha = C.gamma / v;
+  C.alpha_f = (float)C.alpha;
+  C.alpha_x = C.alpha;
+  C.alpha_xf = C.alpha_f;
+  return true;
+}
+
+// |r|^2 = v after an iteration: counts it and decides on a reliable update
+// (do_rel); false: not finite
+__device__ __forceinline__ bool count_update(ColState& C, double v, bool late) {
+  C.rr = v;
+  C.iter += 1;
+  if (!isfinite(v)) return false;
+  if (v <= C.tol2 || v < C.delta2 * C.rr_ref || C.iter >= C.maxiter || late) C.do_rel = 1;
+  else if (C.zr) form_beta(C, v);
+  return true;
+}
+
 // CG scalar recurrences on one column's state, run by one thread.  Where z = r
 // (zr) the update of r, or the reliable update that replaces r, also forms
 // beta: |z|^2 is the sum at hand, and neither a pass over r nor a second
@@ -993,30 +1061,13 @@ __device__ __forceinline__ void finalize(const RedArgs& ra, ColState& C, double 
       }
       break;
     case FIN_ALPHA:
-      if (!C.active) break;
-      if (!(v > 0.0) || !isfinite(v) || !isfinite(C.gamma)) {
-        // p^dag A p <= 0 or not finite: CG cannot continue
-        deactivate(C, ra.flags, 7 /* DW_ERR_BREAKDOWN */);
-      } else {
-        C.alpha = C.gamma / v;
-        C.alpha_f = (float)C.alpha;
-        C.alpha_x = C.alpha;
-        C.alpha_xf = C.alpha_f;
-      }
+      if (C.active && !form_alpha(C, v)) deactivate(C, ra.flags, 7 /* DW_ERR_BREAKDOWN */);
       break;
     case FIN_UPDATE: {
       if (!C.active) break;
-      C.rr = v;
-      C.iter += 1;
-      bool timeout = C.deadline_ns != 0ull && globaltimer_ns() > C.deadline_ns;
-      if (!isfinite(v)) {
-        deactivate(C, ra.flags, 7);
-      } else if (v <= C.tol2 || v < C.delta2 * C.rr_ref || C.iter >= C.maxiter || timeout) {
-        C.do_rel = 1;
-        atomicAdd(&ra.flags->rel_pending, 1);
-      } else if (C.zr) {
-        form_beta(C, v);
-      }
+      const bool late = C.deadline_ns != 0ull && globaltimer_ns() > C.deadline_ns;
+      if (!count_update(C, v, late)) deactivate(C, ra.flags, 7);
+      else if (C.do_rel) atomicAdd(&ra.flags->rel_pending, 1);
       break;
     }
     case FIN_XNORM:
@@ -1098,11 +1149,13 @@ __device__ __forceinline__ DF to_partial(DF v) { return v; }
 __device__ __forceinline__ DF to_partial(double v) { return DF(v); }
 __device__ __forceinline__ DF red_zero(DF) { return df_make(0.f, 0.f); }
 __device__ __forceinline__ double red_zero(double) { return 0.0; }
-// warp total in lane 0, fixed order, double-float on the FP32 pipes
-__device__ __forceinline__ DF warp_sum_lane0(DF v) {
+// warp total in lane 0, fixed order, double-float on the FP32 pipes; from = 4
+// when only lanes 0-7 hold values (adding the others' zeros changes no bit)
+__device__ __forceinline__ DF warp_sum_lane0(DF v, int from = 16) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
+    if (o > from) continue;
     const float th = __shfl_down_sync(0xffffffffu, v.hi, o);
     const float tl = __shfl_down_sync(0xffffffffu, v.lo, o);
     if (lane < o) v = v + df_make(th, tl);
@@ -1195,37 +1248,47 @@ struct FinPlan {
 // Measured at 16^3x32 (512 partials): 4.2 us per launch before, see k_finish's
 // caller for the rule on the block size.
 constexpr int kFinishThreads = 1024, kFinishThreadsSmall = 256;
+// Graph condition set by the last column of a finishing kernel: on = 1 the
+// reliable-update node's, 2 the loop's; 0 none.
 struct RelCond {
   unsigned long long handle;
   int on;
 };
-static __global__ void __launch_bounds__(kFinishThreads) k_finish(const __grid_constant__ FinPlan F, RedArgs ra,
-                                                                  RelCond rel) {
-  __shared__ DF wpart[kFinishThreads / 32];
+// Thread t of n: its share of a column's partials, in order.
+__device__ __forceinline__ DF partial_share(const DF* p, int ntiles, int t, int n) {
+  DF v = df_make(0.f, 0.f);
+  for (int i0 = t; i0 < ntiles; i0 += 8 * n) {
+    float2 q[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int i = i0 + j * n;
+      q[j] = i < ntiles ? __ldcg(reinterpret_cast<const float2*>(p + i)) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (i0 - t + j * n >= ntiles) break;  // past the last partial for every thread
+      v = v + df_make(q[j].x, q[j].y);
+    }
+  }
+  return v;
+}
+template <int N>
+__global__ void __launch_bounds__(N) k_finish(const __grid_constant__ FinPlan F, RedArgs ra, RelCond rel) {
+  __shared__ DF wpart[N / 32];
   const int col = blockIdx.x;
   const int si = F.nrhs == 1 ? col : col / F.nrhs, r = col - si * F.nrhs;
   const int ntiles = F.ntiles[si];
   const DF* p = ra.partial + F.part0[si] + (size_t)r * ntiles;
   ColState C;
   if (threadIdx.x == 0) C = ra.cols[col];
-  DF v = df_make(0.f, 0.f);
-  for (int i0 = threadIdx.x; i0 < ntiles; i0 += 8 * blockDim.x) {
-    float2 t[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int i = i0 + j * blockDim.x;
-      t[j] = i < ntiles ? __ldcg(reinterpret_cast<const float2*>(p + i)) : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) v = v + df_make(t[j].x, t[j].y);
-  }
+  DF v = partial_share(p, ntiles, threadIdx.x, N);
   v = warp_sum_lane0(v);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane == 0) wpart[warp] = v;
   __syncthreads();
   if (warp != 0) return;
-  v = lane < (int)(blockDim.x >> 5) ? wpart[lane] : df_make(0.f, 0.f);
-  v = warp_sum_lane0(v);
+  v = lane < N / 32 ? wpart[lane] : df_make(0.f, 0.f);
+  v = warp_sum_lane0(v, N / 64);
   if (lane != 0) return;
   finalize(ra, C, (double)v);
   ra.cols[col] = C;
@@ -1237,8 +1300,13 @@ static __global__ void __launch_bounds__(kFinishThreads) k_finish(const __grid_c
     }
     if (last) {
       ra.flags->fin_count = 0;
-      const bool run = atomicAdd(&ra.flags->rel_pending, 0) > 0;
-      if (run) ra.flags->rel_runs += 1;
+      bool run;
+      if (rel.on == 1) {
+        run = atomicAdd(&ra.flags->rel_pending, 0) > 0;
+        if (run) ra.flags->rel_runs += 1;
+      } else {
+        run = atomicAdd(&ra.flags->active, 0) > 0 && ra.flags->loops < ra.flags->max_loops;
+      }
       cudaGraphSetConditional(rel.handle, run ? 1u : 0u);
     }
   }

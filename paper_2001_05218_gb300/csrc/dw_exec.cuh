@@ -120,8 +120,10 @@ inline void finish(const Exec& E, int par_mode, int fin, RelCond rel = RelCond{0
     F.ntiles[i] = i < E.P.nsys ? (par_mode == 2 ? 2 * S.tpp : S.tpp) : 0;
     if (F.ntiles[i] > most) most = F.ntiles[i];
   }
-  const int threads = most <= 8 * kFinishThreadsSmall ? kFinishThreadsSmall : kFinishThreads;
-  k_finish<<<E.P.ncols, threads, 0, E.st>>>(F, E.ra(fin), rel);
+  if (most <= 8 * kFinishThreadsSmall)
+    k_finish<kFinishThreadsSmall><<<E.P.ncols, kFinishThreadsSmall, 0, E.st>>>(F, E.ra(fin), rel);
+  else
+    k_finish<kFinishThreads><<<E.P.ncols, kFinishThreads, 0, E.st>>>(F, E.ra(fin), rel);
   if (pr.timing) {
     cudaEventRecord(eb, E.st);
     Profiler::Rec r;
@@ -135,7 +137,8 @@ inline void finish(const Exec& E, int par_mode, int fin, RelCond rel = RelCond{0
 }
 
 template <int SPA, int LP, bool C12, bool DAG, int OP = OP_WILSON, class In, class Epi>
-inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int fin = FIN_STORE0) {
+inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int fin = FIN_STORE0,
+                RelCond rc = RelCond{0, 0}) {
   Profiler& pr = profiler();
   cudaEvent_t ea = nullptr, eb = nullptr;
   if (pr.on) pr.launches += 1;
@@ -154,10 +157,19 @@ inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int 
     launched = true;
   }
   if constexpr ((SPA == P16 || SPA == PB16) && LP == SPA && OP == OP_WILSON && std::is_same<In, InOne<SPA>>::value) {
-    if (E.P.pair && E.P.nrhs >= 2) {  // two right-hand sides per thread, each link loaded once for both
+    if (E.P.pair == 1 && E.P.nrhs >= 2) {  // two right-hand sides per thread, each link loaded once for both
       const unsigned npar = par_mode == 2 ? 2u : 1u;
       const dim3 g(npar * E.P.B.ntot * ((E.P.nrhs + 2 * E.P.B.RB - 1) / (2 * E.P.B.RB)));
       k_hop_pair<SPA, C12, DAG, Epi><<<g, E.P.block, 0, E.st>>>(E.batch(), par_mode, link_slot, in.slot, epi, E.ra(fin));
+      launched = true;
+    }
+  }
+  // FP32 and 16-bit Wilson stencils on small lattices: four threads per site
+  if constexpr (SPA != P64 && SPA != PDF && LP == SPA && OP == OP_WILSON && std::is_same<In, InOne<SPA>>::value) {
+    if (E.P.pair == 2) {
+      const unsigned n = E.P.block.x;
+      k_hop_split<SPA, LP, C12, DAG, In, Epi><<<E.grid(par_mode), 4 * n, n / 32 * (3 * 24 * 32 * sizeof(float)), E.st>>>(
+          E.batch(), par_mode, link_slot, in, epi, E.ra(fin));
       launched = true;
     }
   }
@@ -186,7 +198,7 @@ inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int 
     r.flops = (OP == OP_LAPLACE ? 2280.0 : 1320.0) * sites;
     pr.recs.push_back(r);
   }
-  if (Epi::kReduce) finish(E, par_mode, fin);
+  if (Epi::kReduce) finish(E, par_mode, fin, rc);
 }
 
 template <int SP>

@@ -481,7 +481,7 @@ static std::string device_name() {
   return name;
 }
 std::string tune_key(const dw_lattice* lats, int n, int nrhs, int prec, int c12) {
-  std::string key = device_name() + "/v6/" + prec_name(prec) + (c12 ? "c12" : "c18") + "/r" +
+  std::string key = device_name() + "/v5/" + prec_name(prec) + (c12 ? "c12" : "c18") + "/r" +
                     std::to_string(nrhs);
   for (int i = 0; i < n; ++i)
     key += "/" + std::to_string(lats[i].dims[0]) + "x" + std::to_string(lats[i].dims[1]) + "x" +

@@ -525,9 +525,14 @@ struct EpiXpay {
   template <typename R>
   __device__ __forceinline__ Packed prepare(const SysDesc& S, int par, int r, int s, Cx<R> (&acc)[12],
                                             typename RedT<R>::type& nrm) const {
-    using RO = typename Spin<SPO>::R;
     Cx<typename Spin<SPX>::R> xv[12];
     Spin<SPX>::load(slot_ptr(S, slot_x, r, par), S.vh, s, xv);
+    return form(S, acc, xv, nrm);
+  }
+  template <typename R>
+  __device__ __forceinline__ Packed form(const SysDesc& S, Cx<R> (&acc)[12], const Cx<typename Spin<SPX>::R> (&xv)[12],
+                                         typename RedT<R>::type& nrm) const {
+    using RO = typename Spin<SPO>::R;
     const R c = coef<COEF, R>(S);
     Cx<RO> o[12];
     R n = (R)0;
@@ -848,6 +853,46 @@ __device__ __forceinline__ void laplace_dirs(const SysDesc& S, const In& in, con
   }
 }
 
+// ------------------------------------------------------------------ one direction pair
+// acc += the forward and backward hop along MU at output site s (forward
+// projector sign SF, backward -SF).
+template <int MU, int SPA, int LP, bool C12, int SF, class In, typename R>
+__device__ __forceinline__ void hop_mu(const SysDesc& S, const In& in, const Coord& c, int s, int r, int pin,
+                                       const char* own, const char* nbr, long long mu_stride, Cx<R> (&acc)[12]) {
+  float eta;
+  const int nf = neighbour<MU, +1>(S, c, s, &eta);
+  if constexpr (SPA == P16 || SPA == PB16) {
+    float sc;
+    uint32_t p[12], h[6], u[9];
+    Cx<float> g[6];
+    in.load_words(S, pin, r, nf, p, sc);
+    project_w<MU, SF, SPA>(p, h);
+    Link<LP, C12>::load_words(own + MU * mu_stride, S.vh, s, u);
+    su3_mul_w<false, SPA>(u, h, g);
+    accumulate_w<MU, SF>(acc, g, eta < 0.f ? -sc : sc);
+    const int nb = neighbour<MU, -1>(S, c, s, &eta);
+    in.load_words(S, pin, r, nb, p, sc);
+    project_w<MU, -SF, SPA>(p, h);
+    Link<LP, C12>::load_words(nbr + MU * mu_stride, S.vh, nb, u);
+    su3_mul_w<true, SPA>(u, h, g);
+    accumulate_w<MU, -SF>(acc, g, eta < 0.f ? -sc : sc);
+  } else {
+    Cx<R> p[12], h[6], g[6], u[9];
+    R sc;
+    in.load_raw(S, pin, r, nf, p, sc);
+    project<MU, SF>(p, h);
+    Link<LP, C12>::load(own + MU * mu_stride, S.vh, s, u);
+    su3_mul<false>(u, h, g);
+    accumulate_w<MU, SF>(acc, g, eta < 0.f ? -sc : sc);
+    const int nb = neighbour<MU, -1>(S, c, s, &eta);
+    in.load_raw(S, pin, r, nb, p, sc);
+    project<MU, -SF>(p, h);
+    Link<LP, C12>::load(nbr + MU * mu_stride, S.vh, nb, u);
+    su3_mul<true>(u, h, g);
+    accumulate_w<MU, -SF>(acc, g, eta < 0.f ? -sc : sc);
+  }
+}
+
 // ------------------------------------------------------------------ the stencil kernel
 // par_mode 0/1: output parity fixed, grid = ntot blocks.  par_mode 2: both
 // parities, grid = 2*ntot (block b >= ntot works on odd output sites).
@@ -894,66 +939,22 @@ __global__ void __launch_bounds__(256, HopOccupancy<SPA>::kMinBlocks)
       const char* ulink_nb = slot_ptr(S, link_slot, 0, pin);   // links based at the neighbour
       const long long mu_stride = (long long)Link<LP, C12>::kBytes * S.vh;
       constexpr int SF = DAG ? +1 : -1;  // forward projector sign
-      constexpr int SB = -SF;            // backward projector sign
       Cx<R> acc[12];
 #pragma unroll
       for (int k = 0; k < 12; ++k) acc[k] = cx((R)0, (R)0);
 
-#define DW_HOP_DIR(MU)                                                          \
-  {                                                                             \
-    float eta;                                                                  \
-    Cx<R> p[12], h[6], g[6], u[9];                                              \
-    R sc;                                                                       \
-    const int nf = neighbour<MU, +1>(S, c, s, &eta);                            \
-    in.load_raw(S, pin, r, nf, p, sc);                                          \
-    project<MU, SF>(p, h);                                                      \
-    Link<LP, C12>::load(ulink_own + MU * mu_stride, S.vh, s, u);                 \
-    su3_mul<false>(u, h, g);                                                    \
-    accumulate_w<MU, SF>(acc, g, eta < 0.f ? -sc : sc);                         \
-    const int nb = neighbour<MU, -1>(S, c, s, &eta);                            \
-    in.load_raw(S, pin, r, nb, p, sc);                                          \
-    project<MU, SB>(p, h);                                                      \
-    Link<LP, C12>::load(ulink_nb + MU * mu_stride, S.vh, nb, u);                 \
-    su3_mul<true>(u, h, g);                                                     \
-    accumulate_w<MU, SB>(acc, g, eta < 0.f ? -sc : sc);                         \
-  }
-#define DW_HOP_DIR_W(MU)                                                        \
-  {                                                                             \
-    float eta, sc;                                                              \
-    uint32_t p[12], h[6], u[9];                                                 \
-    Cx<float> g[6];                                                             \
-    const int nf = neighbour<MU, +1>(S, c, s, &eta);                            \
-    in.load_words(S, pin, r, nf, p, sc);                                        \
-    project_w<MU, SF, SPA>(p, h);                                               \
-    Link<LP, C12>::load_words(ulink_own + MU * mu_stride, S.vh, s, u);           \
-    su3_mul_w<false, SPA>(u, h, g);                                             \
-    accumulate_w<MU, SF>(acc, g, eta < 0.f ? -sc : sc);                         \
-    const int nb = neighbour<MU, -1>(S, c, s, &eta);                            \
-    in.load_words(S, pin, r, nb, p, sc);                                        \
-    project_w<MU, SB, SPA>(p, h);                                               \
-    Link<LP, C12>::load_words(ulink_nb + MU * mu_stride, S.vh, nb, u);           \
-    su3_mul_w<true, SPA>(u, h, g);                                              \
-    accumulate_w<MU, SB>(acc, g, eta < 0.f ? -sc : sc);                         \
-  }
       if constexpr (OP == OP_LAPLACE) {
         laplace_dirs<SPA, LP, C12>(S, in, c, s, r, pin, ulink_own, ulink_nb, mu_stride, acc);
         if constexpr (SPA == PDF) {
 #pragma unroll
           for (int k = 0; k < 12; ++k) acc[k] = cx(renorm(acc[k].re), renorm(acc[k].im));
         }
-      } else if constexpr (SPA == P16 || SPA == PB16) {
-        DW_HOP_DIR_W(0)
-        DW_HOP_DIR_W(1)
-        DW_HOP_DIR_W(2)
-        DW_HOP_DIR_W(3)
       } else {
-        DW_HOP_DIR(0)
-        DW_HOP_DIR(1)
-        DW_HOP_DIR(2)
-        DW_HOP_DIR(3)
+        hop_mu<0, SPA, LP, C12, SF>(S, in, c, s, r, pin, ulink_own, ulink_nb, mu_stride, acc);
+        hop_mu<1, SPA, LP, C12, SF>(S, in, c, s, r, pin, ulink_own, ulink_nb, mu_stride, acc);
+        hop_mu<2, SPA, LP, C12, SF>(S, in, c, s, r, pin, ulink_own, ulink_nb, mu_stride, acc);
+        hop_mu<3, SPA, LP, C12, SF>(S, in, c, s, r, pin, ulink_own, ulink_nb, mu_stride, acc);
       }
-#undef DW_HOP_DIR
-#undef DW_HOP_DIR_W
       if constexpr (Epi::kSplit) po = epi.prepare(S, par, r, s, acc, nrm);
       else epi.write(S, par, r, s, acc, nrm);
     }
@@ -964,6 +965,88 @@ __global__ void __launch_bounds__(256, HopOccupancy<SPA>::kMinBlocks)
     } else if constexpr (Epi::kReduce) {
       DW_BLOCK_REDUCE(nrm)
     }
+  }
+}
+
+// ------------------------------------------------------------------ four threads per site
+// The FP32 and 16-bit Wilson stencils on lattices too small to fill the GPU:
+// one warp per mu for 32 consecutive sites, the four partial sums added in
+// shared memory (mu = 0 1 2 3, in that order) by the warp of mu = 0, which
+// runs the epilogue.  With one thread per site a 16^3x32 launch has 13 warps
+// per SM, each a serial chain of eight load latencies; four times the warps
+// with a quarter of the chain hide it.  On large lattices the extra pass
+// through shared memory costs more than it gives (the solver's small_lattices
+// says where the line lies).
+// Blocks: T sites x RB right-hand sides (T RB <= 128), 4 T RB threads, warps
+// (right-hand side, site group, mu).
+template <int SPA, int LP, bool C12, bool DAG, class In, class Epi>
+__global__ void __launch_bounds__(512, 2)
+    k_hop_split(const __grid_constant__ Batch B, int par_mode, int link_slot, In in, Epi epi, RedArgs ra) {
+  using R = typename Spin<SPA>::R;
+  extern __shared__ float parts[];  // [site group][3][24][32]
+  const int T = B.T, RB = B.RB;
+  const unsigned bx = B.rev ? gridDim.x - 1u - blockIdx.x : blockIdx.x;
+  int by = 0, b = (int)bx, par, rl = 0;
+  if (B.ny > 1) {
+    b = (int)(bx / (unsigned)B.ny);
+    by = (int)bx - b * B.ny;
+  }
+  if (par_mode == 2) {
+    par = b >= B.ntot ? 1 : 0;
+    b -= par * B.ntot;
+  } else {
+    par = par_mode;
+  }
+  const SysDesc& S = B.sd[block_system(B, b)];
+  const int lane = threadIdx.x & 31, mu = (threadIdx.x >> 5) & 3, group = threadIdx.x >> 7;
+  if (RB > 1) rl = group / (T >> 5);
+  const int r = by * RB + rl;
+  const int tile = b - S.tile0;
+  const int s = tile * T + ((group - rl * (T >> 5)) << 5) + lane;
+  const bool valid = s < S.vh && r < S.nrhs && gate_of(epi.gate, ra.cols, S.col0 + r);
+  Cx<R> acc[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) acc[k] = cx((R)0, (R)0);
+  if (valid) {
+    const Coord c = coord_of(S, s, par);
+    const int pin = par ^ 1;
+    const char* own = slot_ptr(S, link_slot, 0, par);
+    const char* nbr = slot_ptr(S, link_slot, 0, pin);
+    const long long mu_stride = (long long)Link<LP, C12>::kBytes * S.vh;
+    constexpr int SF = DAG ? +1 : -1;
+    if (mu == 0) hop_mu<0, SPA, LP, C12, SF>(S, in, c, s, r, pin, own, nbr, mu_stride, acc);
+    else if (mu == 1) hop_mu<1, SPA, LP, C12, SF>(S, in, c, s, r, pin, own, nbr, mu_stride, acc);
+    else if (mu == 2) hop_mu<2, SPA, LP, C12, SF>(S, in, c, s, r, pin, own, nbr, mu_stride, acc);
+    else hop_mu<3, SPA, LP, C12, SF>(S, in, c, s, r, pin, own, nbr, mu_stride, acc);
+  }
+  float* mine = parts + (size_t)group * (3 * 24 * 32) + lane;
+  if (mu != 0) {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      mine[((mu - 1) * 24 + 2 * k) * 32] = acc[k].re;
+      mine[((mu - 1) * 24 + 2 * k + 1) * 32] = acc[k].im;
+    }
+  }
+  __syncthreads();
+  typename RedT<R>::type nrm = red_zero(typename RedT<R>::type());
+  typename Epi::Packed po;
+  const bool out = valid && mu == 0;
+  if (out) {
+#pragma unroll
+    for (int m = 0; m < 3; ++m)
+#pragma unroll
+      for (int k = 0; k < 12; ++k)
+        acc[k] = acc[k] + cx(mine[(m * 24 + 2 * k) * 32], mine[(m * 24 + 2 * k + 1) * 32]);
+    if constexpr (Epi::kSplit) po = epi.prepare(S, par, r, s, acc, nrm);
+    else epi.write(S, par, r, s, acc, nrm);
+  }
+  if constexpr (Epi::kReduce) {
+    const int ntiles = par_mode == 2 ? 2 * S.tpp : S.tpp;
+    reduce_block(S, 4 * T, RB, par_mode == 2 ? par * S.tpp + tile : tile, ntiles, nrm, ra, by, [&] {
+      if constexpr (Epi::kSplit) {
+        if (out) epi.commit(S, par, r, s, po);
+      }
+    });
   }
 }
 
@@ -1274,6 +1357,50 @@ __global__ void __launch_bounds__(256, 2)
 }
 
 // ------------------------------------------------------------------ site-local kernels
+// r -= alpha w at one site: the words to store and |r|^2 as stored (the norm is
+// taken of the rounded value, so the recursion sees what the next kernels read)
+template <int SPL>
+__device__ __forceinline__ typename Spin<SPL>::Packed update_r_site(const SysDesc& S, int par, int r, int s,
+                                                                   const ColState& C,
+                                                                   typename RedT<typename Spin<SPL>::R>::type& nrm) {
+  using RL = typename Spin<SPL>::R;
+  Cx<RL> w[12], rv[12];
+  Spin<SPL>::load(slot_ptr(S, S_W, r, par), S.vh, s, w);
+  Spin<SPL>::load(slot_ptr(S, S_R, r, par), S.vh, s, rv);
+  const RL a = scalar_as<RL>(C.alpha, C.alpha_f);
+  RL n = (RL)0;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) rv[k] = cx(fma(-a, w[k].re, rv[k].re), fma(-a, w[k].im, rv[k].im));
+  Spin<SPL>::roundtrip(rv);
+#pragma unroll
+  for (int k = 0; k < 12; ++k) n = fma(rv[k].re, rv[k].re, fma(rv[k].im, rv[k].im, n));
+  nrm = to_red(n);
+  return Spin<SPL>::pack(rv);
+}
+
+// xl += alpha_x p (the increment of the iteration that used p, unless a
+// reliable update has folded it already: alpha_x = 0);  p = z + beta p
+template <int SPL, int SPA>
+__device__ __forceinline__ void update_p_site(const SysDesc& S, int par, int r, int s, const ColState& C) {
+  using RL = typename Spin<SPL>::R;
+  using RA = typename Spin<SPA>::R;
+  const RL beta = scalar_as<RL>(C.beta, C.beta_f);
+  Cx<RL> p[12], z[12];
+  Spin<SPL>::load(slot_ptr(S, S_P, r, par), S.vh, s, p);
+  Spin<SPL>::load(slot_ptr(S, S_Z, r, par), S.vh, s, z);
+  if (C.alpha_x != 0.0) {
+    const RA aa = scalar_as<RA>(C.alpha_x, C.alpha_xf);
+    Cx<RA> xl[12];
+    Spin<SPA>::load(slot_ptr(S, S_XL, r, par), S.vh, s, xl);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) xl[k] = cx(fma(aa, (RA)p[k].re, xl[k].re), fma(aa, (RA)p[k].im, xl[k].im));
+    Spin<SPA>::store(slot_wptr(S, S_XL, r, par), S.vh, s, xl);
+  }
+#pragma unroll
+  for (int k = 0; k < 12; ++k) p[k] = cx(fma(beta, p[k].re, z[k].re), fma(beta, p[k].im, z[k].im));
+  Spin<SPL>::store(slot_wptr(S, S_P, r, par), S.vh, s, p);
+}
+
 // r -= alpha w;  reduction |r|^2 -> FIN_UPDATE.  The matching x-increment
 // xl += alpha p is left to k_update_p (which reads p anyway) or, when a
 // reliable update comes first, to k_fold_x: ColState::alpha_x holds it.
@@ -1283,23 +1410,7 @@ __global__ void __launch_bounds__(256) k_update_r(const __grid_constant__ Batch 
   using RL = typename Spin<SPL>::R;
   typename RedT<RL>::type nrm = red_zero(typename RedT<RL>::type());
   typename Spin<SPL>::Packed rp;
-  if (valid) {
-    const ColState& C = ra.cols[S.col0 + r];
-    Cx<RL> w[12], rv[12];
-    Spin<SPL>::load(slot_ptr(S, S_W, r, par), S.vh, s, w);
-    Spin<SPL>::load(slot_ptr(S, S_R, r, par), S.vh, s, rv);
-    const RL a = scalar_as<RL>(C.alpha, C.alpha_f);
-    RL n = (RL)0;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) rv[k] = cx(fma(-a, w[k].re, rv[k].re), fma(-a, w[k].im, rv[k].im));
-    // the norm is taken of the value as stored, so the recursion sees what
-    // the next kernels will read
-    Spin<SPL>::roundtrip(rv);
-    rp = Spin<SPL>::pack(rv);
-#pragma unroll
-    for (int k = 0; k < 12; ++k) n = fma(rv[k].re, rv[k].re, fma(rv[k].im, rv[k].im, n));
-    nrm = to_red(n);
-  }
+  if (valid) rp = update_r_site<SPL>(S, par, r, s, ra.cols[S.col0 + r], nrm);
   ra.fin = FIN_UPDATE;
   DW_BLOCK_REDUCE_STORE(nrm, [&] {
     if (valid) Spin<SPL>::store_packed(slot_wptr(S, S_R, r, par), S.vh, s, rp);
@@ -1312,8 +1423,7 @@ struct LoopCond {
   int on;
 };
 
-// xl += alpha_x p (the increment of the iteration that used p, unless a
-// reliable update has folded it already: alpha_x = 0);  p = z + beta p
+// xl += alpha_x p;  p = z + beta p (update_p_site)
 template <int SPL, int SPA>
 __global__ void __launch_bounds__(256) k_update_p(const __grid_constant__ Batch B, int par_mode, RedArgs ra,
                                                   LoopCond lc) {
@@ -1325,26 +1435,7 @@ __global__ void __launch_bounds__(256) k_update_p(const __grid_constant__ Batch 
     cudaGraphSetConditional(lc.handle, (ra.flags->active > 0 && loops < ra.flags->max_loops) ? 1u : 0u);
   }
   DW_BLOCK_PROLOGUE(G_ACTIVE)
-  if (valid) {
-    using RL = typename Spin<SPL>::R;
-    using RA = typename Spin<SPA>::R;
-    const ColState& C = ra.cols[S.col0 + r];
-    const RL beta = scalar_as<RL>(C.beta, C.beta_f);
-    Cx<RL> p[12], z[12];
-    Spin<SPL>::load(slot_ptr(S, S_P, r, par), S.vh, s, p);
-    Spin<SPL>::load(slot_ptr(S, S_Z, r, par), S.vh, s, z);
-    if (C.alpha_x != 0.0) {
-      const RA aa = scalar_as<RA>(C.alpha_x, C.alpha_xf);
-      Cx<RA> xl[12];
-      Spin<SPA>::load(slot_ptr(S, S_XL, r, par), S.vh, s, xl);
-#pragma unroll
-      for (int k = 0; k < 12; ++k) xl[k] = cx(fma(aa, (RA)p[k].re, xl[k].re), fma(aa, (RA)p[k].im, xl[k].im));
-      Spin<SPA>::store(slot_wptr(S, S_XL, r, par), S.vh, s, xl);
-    }
-#pragma unroll
-    for (int k = 0; k < 12; ++k) p[k] = cx(fma(beta, p[k].re, z[k].re), fma(beta, p[k].im, z[k].im));
-    Spin<SPL>::store(slot_wptr(S, S_P, r, par), S.vh, s, p);
-  }
+  if (valid) update_p_site<SPL, SPA>(S, par, r, s, ra.cols[S.col0 + r]);
 }
 
 // First residual for a zero initial guess: r_low = src, reduction |src|^2 -> FIN_RESID0

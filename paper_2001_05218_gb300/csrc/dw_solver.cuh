@@ -34,6 +34,7 @@
 #include <chrono>
 
 #include "dw_exec.cuh"
+#include "dw_loop.cuh"
 #include "dw_tune.cuh"
 
 namespace dw {
@@ -43,6 +44,17 @@ enum Mode { MODE_EO = 0, MODE_FULL = 1, MODE_NORMAL = 2, MODE_HERM = 3 };
 inline bool eo_mode(int mode) { return mode == MODE_EO || mode == MODE_HERM; }
 // plain CG: the search direction is built from r itself
 inline bool z_is_r(int mode) { return mode == MODE_NORMAL || mode == MODE_HERM; }
+
+// Sites and right-hand sides of one parity in all.
+inline long long parity_work(const std::vector<dw_lattice>& lats, int nrhs) {
+  long long sites = 0;
+  for (auto& l : lats) sites += vh_of(l) * nrhs;
+  return sites;
+}
+// Small systems run in blocks of 32 sites: up to kSplitSites with four threads
+// per site (k_hop_split), and even-odd systems up to kLoopSites with all
+// iterations in one kernel (k_cg_loop).
+constexpr long long kSplitSites = 16384, kLoopSites = 65536;
 
 struct SolveArgs {
   int n;
@@ -71,7 +83,7 @@ struct CG {
   static constexpr int kLinkLo = S_LLO;
 
   // reliable update (gated by do_rel) and its finalizer
-  static void reliable(const Exec& E, int mode) {
+  static void reliable(const Exec& E, int mode, RelCond rc = RelCond{0, 0}) {
     // even-odd systems: x_e += xl_e (xl_e = 0); t_o = H_oe x_e; r_e = bh - x_e + k^2 H_eo t_o
     // (MODE_HERM: the same with the Laplacian's K)
     auto eo_reliable = [&] {
@@ -80,7 +92,7 @@ struct CG {
       // grid directions alternate: fold forwards, H_oe backwards, H_eo forwards
       // (the next stencil, z's first hop, walks backwards again)
       hop<H, H, false, false, OP>(E.flipped(), 1, kLinkHi, InOne<H>{S_X}, EpiOut<H, C_ONE>{S_RT, G_REL});
-      hop<H, H, false, false, OP>(E, 0, kLinkHi, InOne<H>{S_RT}, EpiResidEO<L, H>{G_REL}, FIN_RELIABLE);
+      hop<H, H, false, false, OP>(E, 0, kLinkHi, InOne<H>{S_RT}, EpiResidEO<L, H>{G_REL}, FIN_RELIABLE, rc);
     };
     if constexpr (OP == OP_LAPLACE) {
       eo_reliable();
@@ -139,6 +151,17 @@ struct CG {
   static dw_status build_graph(const Exec& E, int mode, cudaGraphExec_t* exec, int* body_kernels,
                                int* rel_kernels);
   static dw_status run_stepped(const Exec& E, int mode, int maxiter);
+
+  // The iterations in one kernel (k_cg_loop): even-odd Wilson systems in FP32 or
+  // 16 bits with blocks of 32 sites, few enough columns and tiles for its sums.
+  static constexpr bool kLoop = OP == OP_WILSON && L != P64 && L != PDF;
+  static bool loop_fits(const Plan& P, int mode) {
+    if (!kLoop || mode != MODE_EO || P.B.T != 32 || P.B.RB != 1 || P.ncols > kLoopCols) return false;
+    for (int i = 0; i < P.nsys; ++i)
+      if (P.B.sd[i].tpp > kLoopPartials) return false;
+    return true;
+  }
+  static dw_status launch_loop(const Exec& E, cudaGraphConditionalHandle rel, cudaGraphConditionalHandle loop);
 };
 
 struct CaptureStreams {
@@ -148,6 +171,37 @@ struct CaptureStreams {
     cudaStreamCreateWithFlags(&b, cudaStreamNonBlocking);
   }
 };
+
+template <int L, int A, bool C12, int H, int OP>
+dw_status CG<L, A, C12, H, OP>::launch_loop(const Exec& E, cudaGraphConditionalHandle rel,
+                                            cudaGraphConditionalHandle loop) {
+  if constexpr (kLoop) {
+    // a block takes at least four 32-site items, and one block runs per SM: more
+    // blocks than that only make the barriers dearer
+    int dev = 0, sms = 0;
+    DW_CUDA(cudaGetDevice(&dev));
+    DW_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int items = E.P.B.ntot * E.P.nrhs;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)((items + 3) / 4 < sms ? (items + 3) / 4 : sms));
+    lc.blockDim = dim3(kLoopThreads);
+    lc.stream = E.st;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    count_launch();
+    const RedArgs ra = E.ra(FIN_STORE0);
+    if (E.P.pair == 2)
+      DW_CUDA(cudaLaunchKernelEx(&lc, k_cg_loop<L, A, C12, true>, E.P.B, ra, (unsigned long long)rel,
+                                 (unsigned long long)loop));
+    else
+      DW_CUDA(cudaLaunchKernelEx(&lc, k_cg_loop<L, A, C12, false>, E.P.B, ra, (unsigned long long)rel,
+                                 (unsigned long long)loop));
+  }
+  return DW_OK;
+}
 
 // The whole CG loop as one graph: while (active columns) { iteration with the
 // reliable update in an if-node }.  Both conditions are set on the device, by
@@ -185,10 +239,15 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, int mode, cudaGraphE
   const long long c0 = pr.launches;
   long long c1 = c0, c2 = c0;
   DW_CUDA(cudaStreamBeginCaptureToGraph(cs.a, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-  wstep(E, mode);
-  count_launch();
-  k_update_r<L><<<E.grid(pm), E.P.block, 0, E.st>>>(E.P.B, pm, E.ra(FIN_UPDATE));
-  finish(E, pm, FIN_UPDATE, RelCond{(unsigned long long)hr, 1});
+  const bool one = loop_fits(E.P, mode);
+  if (one) {
+    DW_TRY(launch_loop(E, hr, hw));
+  } else {
+    wstep(E, mode);
+    count_launch();
+    k_update_r<L><<<E.grid(pm), E.P.block, 0, E.st>>>(E.P.B, pm, E.ra(FIN_UPDATE));
+    finish(E, pm, FIN_UPDATE, RelCond{(unsigned long long)hr, 1});
+  }
   {
     cudaStreamCaptureStatus cst;
     cudaGraph_t capg;
@@ -208,15 +267,17 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, int mode, cudaGraphE
     c1 = pr.launches;
     DW_CUDA(cudaStreamBeginCaptureToGraph(cs.b, ip.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                           cudaStreamCaptureModeThreadLocal));
-    reliable(R, mode);
+    reliable(R, mode, one ? RelCond{(unsigned long long)hw, 2} : RelCond{0, 0});
     cudaGraph_t tmp;
     DW_CUDA(cudaStreamEndCapture(cs.b, &tmp));
     c2 = pr.launches;
   }
-  zstep(E, mode, FIN_BETA);
-  k_update_p<L, A><<<E.grid(pm), E.P.block, 0, E.st>>>(E.flipped().batch(), pm, E.ra(FIN_STORE0),
-                                                       LoopCond{(unsigned long long)hw, 1});
-  count_launch();
+  if (!one) {
+    zstep(E, mode, FIN_BETA);
+    k_update_p<L, A><<<E.grid(pm), E.P.block, 0, E.st>>>(E.flipped().batch(), pm, E.ra(FIN_STORE0),
+                                                         LoopCond{(unsigned long long)hw, 1});
+    count_launch();
+  }
   cudaGraph_t tmp;
   DW_CUDA(cudaStreamEndCapture(cs.a, &tmp));
   cudaError_t e = cudaGraphInstantiate(&ge, g, 0);
@@ -312,6 +373,11 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
     Exec& F = fresh.E;
     BlockShape shape{a.p.tile, a.p.tile > 0 ? 1 : 0};
     if (a.p.tile <= 0) shape = tune_inner_shape<L, C12>(lats, nrhs, lo_links, st);
+    if (a.p.tile <= 0 && OP == OP_WILSON && L != P64 && L != PDF) {
+      const long long work = parity_work(lats, nrhs);
+      if (work <= kSplitSites) shape = BlockShape{32, 1, 2};
+      else if (mode == MODE_EO && work <= kLoopSites && n * nrhs <= kLoopCols) shape = BlockShape{32, 1, 0};
+    }
     make_plan(F.P, lats, nrhs, shape.T, shape.RB);
     F.P.pair = shape.pair;
     auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
@@ -502,6 +568,7 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
   cudaEventDestroy(ev0);
   cudaEventDestroy(ev1);
   DW_CUDA(cudaGetLastError());
+  if (hf.bar_error) return set_error(DW_ERR_CUDA, "a grid barrier of the CG loop gave up waiting");
 
   // ---- statistics
   dw_status worst = DW_OK;
