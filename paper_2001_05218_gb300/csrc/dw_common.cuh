@@ -1061,10 +1061,10 @@ __device__ __forceinline__ void finalize(const RedArgs& ra, ColState& C, double 
       }
       break;
     case FIN_ALPHA:
-      if (C.active && !form_alpha(C, v)) deactivate(C, ra.flags, 7 /* DW_ERR_BREAKDOWN */);
+      if (C.active && !C.do_rel && !form_alpha(C, v)) deactivate(C, ra.flags, 7 /* DW_ERR_BREAKDOWN */);
       break;
     case FIN_UPDATE: {
-      if (!C.active) break;
+      if (!C.active || C.do_rel) break;
       const bool late = C.deadline_ns != 0ull && globaltimer_ns() > C.deadline_ns;
       if (!count_update(C, v, late)) deactivate(C, ra.flags, 7);
       else if (C.do_rel) atomicAdd(&ra.flags->rel_pending, 1);
@@ -1110,7 +1110,7 @@ __device__ __forceinline__ void finalize(const RedArgs& ra, ColState& C, double 
       C.beta_f = 0.f;
       break;
     case FIN_BETA:
-      if (!C.active) break;
+      if (!C.active || C.do_rel) break;
       form_beta(C, v);
       break;
   }
@@ -1248,8 +1248,9 @@ struct FinPlan {
 // Measured at 16^3x32 (512 partials): 4.2 us per launch before, see k_finish's
 // caller for the rule on the block size.
 constexpr int kFinishThreads = 1024, kFinishThreadsSmall = 256;
-// Graph condition set by the last column of a finishing kernel: on = 1 the
-// reliable-update node's, 2 the loop's; 0 none.
+// What the last column of a finishing kernel inside the graph does: on = 1 sets
+// the reliable-update node's condition; 2 and 3 count a reliable update, and 2
+// also sets the loop's condition.
 struct RelCond {
   unsigned long long handle;
   int on;
@@ -1300,14 +1301,14 @@ __global__ void __launch_bounds__(N) k_finish(const __grid_constant__ FinPlan F,
     }
     if (last) {
       ra.flags->fin_count = 0;
-      bool run;
       if (rel.on == 1) {
-        run = atomicAdd(&ra.flags->rel_pending, 0) > 0;
-        if (run) ra.flags->rel_runs += 1;
+        cudaGraphSetConditional(rel.handle, atomicAdd(&ra.flags->rel_pending, 0) > 0 ? 1u : 0u);
       } else {
-        run = atomicAdd(&ra.flags->active, 0) > 0 && ra.flags->loops < ra.flags->max_loops;
+        ra.flags->rel_runs += 1;
+        if (rel.on == 2)
+          cudaGraphSetConditional(
+              rel.handle, atomicAdd(&ra.flags->active, 0) > 0 && ra.flags->loops < ra.flags->max_loops ? 1u : 0u);
       }
-      cudaGraphSetConditional(rel.handle, run ? 1u : 0u);
     }
   }
 }

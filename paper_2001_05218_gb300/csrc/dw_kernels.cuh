@@ -57,11 +57,15 @@ __device__ __forceinline__ R scalar_as(double v, float vf) {
   else return DF(v);
 }
 
-__device__ __forceinline__ int gate_of(int g, const ColState* cols, int col) {
+// G_ACTIVE is shut while the column's reliable update is due: what is left of an
+// unrolled pass of the loop does nothing.
+__device__ __forceinline__ int gate_of(int g, const RedArgs& ra, int col) {
   if (g == G_ALL) return 1;
-  if (g == G_XZERO) return cols[col].xzero;
-  if (g == G_ZSRC) return cols[col].zsrc;
-  return g == G_ACTIVE ? cols[col].active : cols[col].do_rel;
+  const ColState& C = ra.cols[col];
+  if (g == G_XZERO) return C.xzero;
+  if (g == G_ZSRC) return C.zsrc;
+  if (g == G_REL) return C.do_rel;
+  return C.active & (C.do_rel ^ 1);
 }
 
 // a + S*b,  S = +1 or -1 (compile time)
@@ -754,7 +758,7 @@ struct EpiResidFull {
   const int r = by * RB + rl;                                              \
   const int tile = b - S.tile0;                                            \
   const int s = tile * T + ((int)threadIdx.x - rl * T);                    \
-  const bool valid = s < S.vh && r < S.nrhs && gate_of(GATE, ra.cols, S.col0 + r);
+  const bool valid = s < S.vh && r < S.nrhs && gate_of(GATE, ra, S.col0 + r);
 
 #define DW_BLOCK_REDUCE(val)                                               \
   {                                                                        \
@@ -1003,7 +1007,7 @@ __global__ void __launch_bounds__(512, 2)
   const int r = by * RB + rl;
   const int tile = b - S.tile0;
   const int s = tile * T + ((group - rl * (T >> 5)) << 5) + lane;
-  const bool valid = s < S.vh && r < S.nrhs && gate_of(epi.gate, ra.cols, S.col0 + r);
+  const bool valid = s < S.vh && r < S.nrhs && gate_of(epi.gate, ra, S.col0 + r);
   Cx<R> acc[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) acc[k] = cx((R)0, (R)0);
@@ -1207,7 +1211,7 @@ __global__ void DW_ROWS_ATTR
   // a warp works on one right-hand side: the gate is the same for all its
   // lanes, and lanes past the last site repeat site 0 without storing
   typename RedT<R>::type nrm = red_zero(typename RedT<R>::type());
-  if (r < S.nrhs && gate_of(epi.gate, ra.cols, S.col0 + r)) {
+  if (r < S.nrhs && gate_of(epi.gate, ra, S.col0 + r)) {
     const int s = ok ? s0 : 0;
     const Coord c = coord_of(S, s, par);
     const int pin = par ^ 1;
@@ -1288,8 +1292,8 @@ __global__ void __launch_bounds__(256, 2)
   const int tile = b - S.tile0;
   const int s = tile * T + (threadIdx.x - rl * T);
   const bool site = s < S.vh;
-  const bool v0 = site && r0 < S.nrhs && gate_of(epi.gate, ra.cols, S.col0 + r0);
-  const bool v1 = site && r1 < S.nrhs && gate_of(epi.gate, ra.cols, S.col0 + r1);
+  const bool v0 = site && r0 < S.nrhs && gate_of(epi.gate, ra, S.col0 + r0);
+  const bool v1 = site && r1 < S.nrhs && gate_of(epi.gate, ra, S.col0 + r1);
   const int r1l = r1 < S.nrhs ? r1 : r0;  // a missing second column reloads the first
   typename RedT<float>::type nrm[2] = {red_zero(typename RedT<float>::type()), red_zero(typename RedT<float>::type())};
   typename Epi::Packed po0, po1;

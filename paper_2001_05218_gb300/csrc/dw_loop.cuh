@@ -261,7 +261,6 @@ __global__ void __launch_bounds__(kLoopThreads, 1)
       f->rel_pending = wanted;
       f->loops += 1;
       f->bar_base = round;
-      if (wanted > 0) f->rel_runs += 1;
       // with a reliable update pending its finishing kernel decides anew
       cudaGraphSetConditional(rel, wanted > 0 ? 1u : 0u);
       cudaGraphSetConditional(loop, active > 0 && f->loops < f->max_loops ? 1u : 0u);

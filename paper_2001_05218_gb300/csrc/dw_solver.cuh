@@ -102,14 +102,14 @@ struct CG {
       count_launch();
       k_fold_x<L, A, H><<<E.grid(2), E.P.block, 0, E.st>>>(E.P.B, 2, E.ra(FIN_STORE0));
       hop<H, H, false, false, OP>(E, 2, kLinkHi, InOne<H>{S_X}, EpiResidFull<L, true, H>{G_REL, S_RT, S_X, S_B},
-                              FIN_RELIABLE);
+                              FIN_RELIABLE, rc);
     } else {
       count_launch();
       k_fold_x<L, A, H><<<E.grid(2), E.P.block, 0, E.st>>>(E.P.B, 2, E.ra(FIN_STORE0));
       // t = D x ; r = b - D^dag t
       hop<H, H, false, false, OP>(E, 2, kLinkHi, InOne<H>{S_X}, EpiXpay<H, H, C_MK, false>{S_AUX0, S_X, G_REL});
       hop<H, H, false, true, OP>(E, 2, kLinkHi, InOne<H>{S_AUX0}, EpiResidFull<L, true, H>{G_REL, S_RT, S_AUX0, S_B},
-                             FIN_RELIABLE);
+                             FIN_RELIABLE, rc);
     }
   }
 
@@ -243,10 +243,24 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, int mode, cudaGraphE
   if (one) {
     DW_TRY(launch_loop(E, hr, hw));
   } else {
-    wstep(E, mode);
-    count_launch();
-    k_update_r<L><<<E.grid(pm), E.P.block, 0, E.st>>>(E.P.B, pm, E.ra(FIN_UPDATE));
-    finish(E, pm, FIN_UPDATE, RelCond{(unsigned long long)hr, 1});
+    // A pass of the while node and the test of the if node cost about 4 us each
+    // (empty kernels in such a graph: 4.5 us per pass, 8.0 with the if node, 0.6
+    // per kernel).  One small column runs four iterations per pass; when one of
+    // them asks for a reliable update the rest of the pass is held.  With larger
+    // grids the held launches cost more than the passes saved, and with several
+    // columns they come too often.
+    const int per_pass = E.P.ncols == 1 && E.grid(pm).x <= 2048 ? 4 : 1;
+    for (int k = 0; k < per_pass; ++k) {
+      if (k > 0) {
+        zstep(E, mode, FIN_BETA);
+        count_launch();
+        k_update_p<L, A><<<E.grid(pm), E.P.block, 0, E.st>>>(E.flipped().batch(), pm, E.ra(FIN_STORE0), LoopCond{0, 0});
+      }
+      wstep(E, mode);
+      count_launch();
+      k_update_r<L><<<E.grid(pm), E.P.block, 0, E.st>>>(E.P.B, pm, E.ra(FIN_UPDATE));
+      finish(E, pm, FIN_UPDATE, RelCond{(unsigned long long)hr, 1});
+    }
   }
   {
     cudaStreamCaptureStatus cst;
@@ -267,7 +281,7 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, int mode, cudaGraphE
     c1 = pr.launches;
     DW_CUDA(cudaStreamBeginCaptureToGraph(cs.b, ip.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                           cudaStreamCaptureModeThreadLocal));
-    reliable(R, mode, one ? RelCond{(unsigned long long)hw, 2} : RelCond{0, 0});
+    reliable(R, mode, one ? RelCond{(unsigned long long)hw, 2} : RelCond{0, 3});
     cudaGraph_t tmp;
     DW_CUDA(cudaStreamEndCapture(cs.b, &tmp));
     c2 = pr.launches;
