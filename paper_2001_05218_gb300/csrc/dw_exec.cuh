@@ -87,6 +87,7 @@ struct Exec {
 struct SolveCacheEntry {
   std::vector<unsigned long long> key;
   Exec E;
+  Exec EH;  // the plan of the high-precision stencils: the same slots and buffers
   char* arena = nullptr;
   cudaGraphExec_t exec = nullptr;
   int body_k = 0, rel_k = 0;
@@ -136,6 +137,12 @@ inline void finish(const Exec& E, int par_mode, int fin, RelCond rel = RelCond{0
   }
 }
 
+// More than 48 KiB of dynamic shared memory for a kernel on the current device.
+template <class K>
+inline void allow_shared(K* kernel, size_t bytes) {
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 template <int SPA, int LP, bool C12, bool DAG, int OP = OP_WILSON, class In, class Epi>
 inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int fin = FIN_STORE0,
                 RelCond rc = RelCond{0, 0}) {
@@ -152,8 +159,10 @@ inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int 
       (SPA == P64 || SPA == PDF) && LP == SPA && OP == OP_WILSON && std::is_same<In, InOne<SPA>>::value;
   bool launched = false;
   if constexpr (kRows) {
-    k_hop_rows<SPA, C12, DAG, Epi><<<E.grid(par_mode), 2 * E.P.block.x, 0, E.st>>>(E.batch(), par_mode, link_slot,
-                                                                                  in.slot, epi, E.ra(fin));
+    const size_t smem = SPA == PDF ? (size_t)E.P.block.x / 16 * RowRing<C12>::kBytes : 0;
+    if (smem > 48 * 1024) allow_shared(k_hop_rows<SPA, C12, DAG, Epi>, smem);
+    k_hop_rows<SPA, C12, DAG, Epi><<<E.grid(par_mode), 2 * E.P.block.x, smem, E.st>>>(
+        E.batch(), par_mode, link_slot, in.slot, epi, E.ra(fin));
     launched = true;
   }
   if constexpr ((SPA == P16 || SPA == PB16) && LP == SPA && OP == OP_WILSON && std::is_same<In, InOne<SPA>>::value) {

@@ -1,6 +1,7 @@
 // dw_field.cu -- field handles, host/device transfers and the layout kernels
 // that convert between the canonical (lexicographic, site-major complex128)
 // order and the even-odd structure-of-arrays storage.
+#include <atomic>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -465,27 +466,35 @@ static void tune_load_once() {
 }
 // A device's name, asked for once: cudaGetDeviceProperties costs microseconds
 // and every operator application looks its block shape up.
-static std::string device_name() {
-  static std::mutex mu;
-  static std::map<int, std::string> names;
+static const std::string& device_name() {
+  static std::atomic<const std::string*> names[64];
+  static const std::string unknown = "gpu";
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return "gpu";
-  std::lock_guard<std::mutex> lock(mu);
-  std::string& name = names[dev];
-  if (name.empty()) {
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return unknown;
+  const std::string* name = names[dev].load(std::memory_order_acquire);
+  if (name == nullptr) {
     cudaDeviceProp prop;
-    name = cudaGetDeviceProperties(&prop, dev) == cudaSuccess ? prop.name : "gpu";
-    for (char& c : name)
+    std::string* fresh = new std::string(cudaGetDeviceProperties(&prop, dev) == cudaSuccess ? prop.name : "gpu");
+    for (char& c : *fresh)
       if (c == ' ') c = '_';
+    if (names[dev].compare_exchange_strong(name, fresh)) name = fresh;
+    else delete fresh;
   }
-  return name;
+  return *name;
 }
 std::string tune_key(const dw_lattice* lats, int n, int nrhs, int prec, int c12) {
-  std::string key = device_name() + "/v5/" + prec_name(prec) + (c12 ? "c12" : "c18") + "/r" +
-                    std::to_string(nrhs);
+  std::string key;
+  key.reserve(64 + 24 * (size_t)n);
+  key += device_name();
+  key += "/v5/";
+  key += prec_name(prec);
+  key += c12 ? "c12/r" : "c18/r";
+  key += std::to_string(nrhs);
   for (int i = 0; i < n; ++i)
-    key += "/" + std::to_string(lats[i].dims[0]) + "x" + std::to_string(lats[i].dims[1]) + "x" +
-           std::to_string(lats[i].dims[2]) + "x" + std::to_string(lats[i].dims[3]);
+    for (int m = 0; m < 4; ++m) {
+      key += m == 0 ? '/' : 'x';
+      key += std::to_string(lats[i].dims[m]);
+    }
   return key;
 }
 bool tune_lookup(const std::string& key, BlockShape* out) {
@@ -701,14 +710,15 @@ dw_status dw_field_export(const dw_field* f, double* dev, dw_stream_t stream) {
 // reserved between calls so that repeated transfers do not reallocate.
 static constexpr uint64_t kStagingKeep = 8ull << 30;
 static std::mutex g_pool_mu;
-static cudaMemPool_t g_pool[64];
+static std::atomic<cudaMemPool_t> g_pool[64];
 
 static dw_status staging_pool(cudaMemPool_t* out) {
   int dev = 0;
   DW_CUDA(cudaGetDevice(&dev));
   DW_CHECK(dev >= 0 && dev < 64, DW_ERR_ARG, "device index %d out of range", dev);
+  if ((*out = g_pool[dev].load(std::memory_order_acquire)) != nullptr) return DW_OK;
   std::lock_guard<std::mutex> lock(g_pool_mu);
-  if (!g_pool[dev]) {
+  if (!g_pool[dev].load()) {
     cudaMemPoolProps props;
     memset(&props, 0, sizeof props);
     props.allocType = cudaMemAllocationTypePinned;
@@ -718,9 +728,9 @@ static dw_status staging_pool(cudaMemPool_t* out) {
     DW_CUDA(cudaMemPoolCreate(&p, &props));
     uint64_t keep = kStagingKeep;
     DW_CUDA(cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep));
-    g_pool[dev] = p;
+    g_pool[dev].store(p, std::memory_order_release);
   }
-  *out = g_pool[dev];
+  *out = g_pool[dev].load();
   return DW_OK;
 }
 

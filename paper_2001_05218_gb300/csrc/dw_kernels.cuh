@@ -1129,43 +1129,91 @@ __device__ __forceinline__ void row_project(const char* in, int vh, int n, int r
   }
 }
 
-// Both directions of one mu for one row.  With g_f = U h_f and g_b = U^dag h_b
-// the upper spin takes g_f + g_b and the lower spin d (g_f - g_b), d the unit
-// factor of the forward projector (the backward one is its negative).
-template <int SPA, bool C12, bool IMAG, typename R>
+// IEEE FP64: both directions of one mu for one row.  With g_f = U h_f and
+// g_b = U^dag h_b the upper spin takes g_f + g_b and the lower spin d (g_f - g_b),
+// d the unit factor of the forward projector (the backward one is its negative).
+// The FP64 pipe (64 cycles per warp instruction) is the bound, so additions are
+// saved: the backward product's chain starts from g_f and yields A = g_f + g_b
+// at no extra cost, and g_f - g_b = 2 g_f - A is one FMA: 18 instead of 24
+// operations per mu and row, none onto empty sums.
+template <bool C12, bool IMAG>
 __device__ __forceinline__ void row_mu(const SysDesc& S, const char* in, const char* own, const char* nbr, int s, int nf,
                                        int nb, int row, int partner, uint32_t cm, uint32_t dm, uint32_t bf, uint32_t bb,
-                                       Cx<R> (&up)[3], Cx<R> (&low)[3], bool first_up, bool first_low) {
-  Cx<R> h[3], g[3], u[9];
-  row_project<SPA, IMAG>(in, S.vh, nf, row, partner, cm, bf, h);
-  Link<SPA, C12>::load(own, S.vh, s, u);
+                                       Cx<double> (&up)[3], Cx<double> (&low)[3], bool first) {
+  Cx<double> h[3], g[3], u[9];
+  row_project<P64, IMAG>(in, S.vh, nf, row, partner, cm, bf, h);
+  Link<P64, C12>::load(own, S.vh, s, u);
   su3_mul_row<false>(u, h, g);
-  row_project<SPA, IMAG>(in, S.vh, nb, row, partner, cm ^ 0x80000000u, bb, h);
-  Link<SPA, C12>::load(nbr, S.vh, nb, u);
-  if constexpr (SPA == P64) {
-    // The FP64 pipe (64 cycles per warp instruction) is the bound, so additions
-    // are saved: the backward product's chain starts from g_f and yields
-    // A = g_f + g_b at no extra cost, and g_f - g_b = 2 g_f - A is one FMA:
-    // 18 instead of 24 operations per mu and row, none onto empty sums.
+  row_project<P64, IMAG>(in, S.vh, nb, row, partner, cm ^ 0x80000000u, bb, h);
+  Link<P64, C12>::load(nbr, S.vh, nb, u);
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      Cx<R> t = cjmadd(u[0 * 3 + a], h[0], g[a]);
-      t = cjmadd(u[1 * 3 + a], h[1], t);
-      t = cjmadd(u[2 * 3 + a], h[2], t);
-      const Cx<R> d = times_unit<IMAG>(cx(fma(2.0, g[a].re, -t.re), fma(2.0, g[a].im, -t.im)), dm);
-      up[a] = first_up ? t : up[a] + t;
-      low[a] = first_low ? d : low[a] + d;
+  for (int a = 0; a < 3; ++a) {
+    Cx<double> t = cjmadd(u[0 * 3 + a], h[0], g[a]);
+    t = cjmadd(u[1 * 3 + a], h[1], t);
+    t = cjmadd(u[2 * 3 + a], h[2], t);
+    const Cx<double> d = times_unit<IMAG>(cx(fma(2.0, g[a].re, -t.re), fma(2.0, g[a].im, -t.im)), dm);
+    up[a] = first ? t : up[a] + t;
+    low[a] = first ? d : low[a] + d;
+  }
+}
+
+// Double-float: the operands of one direction for a warp's 16 sites go through
+// shared memory, copied asynchronously while the direction before is computed
+// (two stages, private to the warp).  A direction is about 480 instructions per
+// thread and its loads about 1 us away; in registers there is no room to hold
+// the next direction's 15 words of 16 bytes at 128 registers per thread.
+// Stage: 12 spinor planes, then the link's planes, 16 sites x 16 bytes each.
+template <bool C12>
+struct RowRing {
+  static constexpr int kChunks = 12 + (C12 ? 6 : 9);
+  static constexpr int kStage = kChunks * 256;  // bytes
+  static constexpr int kBytes = 2 * kStage;     // per warp
+  // lanes j and j + 16 copy the even and the odd planes of site j
+  __device__ static __forceinline__ void issue(char* stage, const char* in, const char* lb, int vh, int n, int li) {
+    const int lane = threadIdx.x & 31, half = lane >> 4;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(stage) + half * 256 + (lane & 15) * 16;
+    const char* p = in + ((size_t)half * vh + n) * 16;
+    const char* q = lb + ((size_t)half * vh + li) * 16;
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + i * 512), "l"(p + (size_t)(2 * i) * vh * 16)
+                   : "memory");
+#pragma unroll
+    for (int i = 0; i < (kChunks - 12 + 1) / 2; ++i)
+      if (2 * i + half < kChunks - 12)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + (6 + i) * 512),
+                     "l"(q + (size_t)(2 * i) * vh * 16)
+                     : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  __device__ static __forceinline__ Cx<DF> word(const char* stage, int chunk) {
+    const float4 t = *reinterpret_cast<const float4*>(stage + chunk * 256 + (threadIdx.x & 15) * 16);
+    return cx(df_make(t.x, t.y), df_make(t.z, t.w));
+  }
+  // one direction for one row: h projected, g = U h (or U^dag h), added up
+  template <bool IMAG, bool ADJ>
+  __device__ static __forceinline__ void direction(const char* stage, int row, int partner, uint32_t cm, uint32_t dm,
+                                                   uint32_t bm, Cx<DF> (&up)[3], Cx<DF> (&low)[3]) {
+    Cx<DF> h[3], g[3], u[9];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      h[c] = row_add(word(stage, 3 * row + c), times_unit<IMAG>(word(stage, 3 * partner + c), cm));
+      h[c] = cx(flip(h[c].re, bm), flip(h[c].im, bm));
     }
-  } else {
-    Cx<R> gb[3];
-    su3_mul_row<true>(u, h, gb);
+#pragma unroll
+    for (int k = 0; k < kChunks - 12; ++k) u[k] = word(stage, 12 + k);
+    if (C12) rebuild_row2(u);
+    su3_mul_row<ADJ>(u, h, g);
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      up[a] = row_add(row_add(up[a], g[a]), gb[a]);
+      up[a] = row_add(up[a], g[a]);
       low[a] = row_add(low[a], times_unit<IMAG>(g[a], dm));
-      low[a] = row_add(low[a], times_unit<IMAG>(gb[a], dm ^ 0x80000000u));
     }
   }
+};
+// The neighbour of a direction (0-7: mu = d / 2, forward for even d).
+__device__ __forceinline__ int neighbour_dir(const SysDesc& S, const Coord& c, int s, int d, float* eta) {
+  return neighbour_rt(S, c, s, d >> 1, (d & 1) ? -1 : +1, eta);
 }
 
 // The FP64-class Wilson stencils (IEEE FP64 and double-float): two threads per
@@ -1179,11 +1227,8 @@ __device__ __forceinline__ void row_mu(const SysDesc& S, const char* in, const c
 //   x: c = -s i, d = s i (both rows)   y: c = d = -s (row 0), s (row 1)
 //   t: c = s, d = s (both rows)        z: c = -s i, d = s i (row 0), the opposite (row 1)
 // Blocks: T sites x RB right-hand sides, 2 T RB threads.
-#ifndef DW_ROWS_ATTR
-#define DW_ROWS_ATTR __launch_bounds__(512, 1)
-#endif
 template <int SPA, bool C12, bool DAG, class Epi>
-__global__ void DW_ROWS_ATTR
+__global__ void __launch_bounds__(512, 1)
     k_hop_rows(const __grid_constant__ Batch B, int par_mode, int link_slot, int in_slot, Epi epi, RedArgs ra) {
   static_assert(SPA == P64 || SPA == PDF, "two threads per site: FP64-class storage");
   using R = typename Spin<SPA>::R;
@@ -1226,27 +1271,68 @@ __global__ void DW_ROWS_ATTR
     for (int k = 0; k < 3; ++k) up[k] = low[k] = cx((R)0, (R)0);
     // x and y, then z and t: one copy of the code for both halves, which keeps
     // the kernel inside the instruction cache
+    if constexpr (SPA == PDF) {
+      using Ring = RowRing<C12>;
+      extern __shared__ char ring_[];
+      char* stage = ring_ + (threadIdx.x >> 5) * Ring::kBytes;
+      float eta;
+      int n = neighbour_dir(S, c, s, 0, &eta);
+      Ring::issue(stage, in, own, S.vh, n, s);
+      uint32_t bm = 0u;  // boundary sign of the direction in the current stage
 #pragma unroll 1
-    for (int ph = 0; ph < 2; ++ph) {
-      const int partner = ph == 0 ? 3 - row : 2 + row;
-      float ef, eb;
-      int nf = ph == 0 ? neighbour<0, +1>(S, c, s, &ef) : neighbour<2, +1>(S, c, s, &ef);
-      int nb = ph == 0 ? neighbour<0, -1>(S, c, s, &eb) : neighbour<2, -1>(S, c, s, &eb);
-      const uint32_t mi = kS ^ (ph == 0 ? 0u : row1);
-      row_mu<SPA, C12, true>(S, in, own, nbr, s, nf, nb, row, partner, mi ^ 0x80000000u, mi, 0u, 0u, up, low, ph == 0,
-                             ph == 0);
-      own += mu_stride;
-      nbr += mu_stride;
-      nf = ph == 0 ? neighbour<1, +1>(S, c, s, &ef) : neighbour<3, +1>(S, c, s, &ef);
-      nb = ph == 0 ? neighbour<1, -1>(S, c, s, &eb) : neighbour<3, -1>(S, c, s, &eb);
-      const uint32_t mr = kS ^ (ph == 0 ? row1 ^ 0x80000000u : 0u);
-      row_mu<SPA, C12, false>(S, in, own, nbr, s, nf, nb, row, partner, mr, mr, __float_as_uint(ef) & 0x80000000u,
-                              __float_as_uint(eb) & 0x80000000u, up, low, false, false);
-      own += mu_stride;
-      nbr += mu_stride;
-      if (ph == 0) {
+      for (int ph = 0; ph < 2; ++ph) {
+        const int partner = ph == 0 ? 3 - row : 2 + row;
+        const uint32_t mi = kS ^ (ph == 0 ? 0u : row1), mr = kS ^ (ph == 0 ? row1 ^ 0x80000000u : 0u);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) low[k] = other_row(low[k]);
+        for (int k = 0; k < 4; ++k) {
+          const int d = 4 * ph + k;
+          uint32_t next_bm = 0u;
+          __syncwarp();  // the stage about to be refilled has been read
+          if (k < 3 || ph == 0) {
+            n = neighbour_dir(S, c, s, d + 1, &eta);
+            next_bm = __float_as_uint(eta) & 0x80000000u;
+            const bool back = (k + 1) & 1;
+            Ring::issue(stage + ((k + 1) & 1) * Ring::kStage, in, (back ? nbr : own) + ((d + 1) >> 1) * mu_stride, S.vh, n,
+                        back ? n : s);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+          } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+          }
+          __syncwarp();
+          const char* st = stage + (k & 1) * Ring::kStage;
+          if (k == 0) Ring::template direction<true, false>(st, row, partner, mi ^ 0x80000000u, mi, 0u, up, low);
+          else if (k == 1) Ring::template direction<true, true>(st, row, partner, mi, mi ^ 0x80000000u, 0u, up, low);
+          else if (k == 2) Ring::template direction<false, false>(st, row, partner, mr, mr, bm, up, low);
+          else Ring::template direction<false, true>(st, row, partner, mr ^ 0x80000000u, mr ^ 0x80000000u, bm, up, low);
+          bm = next_bm;
+        }
+        if (ph == 0) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) low[k] = other_row(low[k]);
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int ph = 0; ph < 2; ++ph) {
+        const int partner = ph == 0 ? 3 - row : 2 + row;
+        float ef, eb;
+        int nf = ph == 0 ? neighbour<0, +1>(S, c, s, &ef) : neighbour<2, +1>(S, c, s, &ef);
+        int nb = ph == 0 ? neighbour<0, -1>(S, c, s, &eb) : neighbour<2, -1>(S, c, s, &eb);
+        const uint32_t mi = kS ^ (ph == 0 ? 0u : row1);
+        row_mu<C12, true>(S, in, own, nbr, s, nf, nb, row, partner, mi ^ 0x80000000u, mi, 0u, 0u, up, low, ph == 0);
+        own += mu_stride;
+        nbr += mu_stride;
+        nf = ph == 0 ? neighbour<1, +1>(S, c, s, &ef) : neighbour<3, +1>(S, c, s, &ef);
+        nb = ph == 0 ? neighbour<1, -1>(S, c, s, &eb) : neighbour<3, -1>(S, c, s, &eb);
+        const uint32_t mr = kS ^ (ph == 0 ? row1 ^ 0x80000000u : 0u);
+        row_mu<C12, false>(S, in, own, nbr, s, nf, nb, row, partner, mr, mr, __float_as_uint(ef) & 0x80000000u,
+                           __float_as_uint(eb) & 0x80000000u, up, low, false);
+        own += mu_stride;
+        nbr += mu_stride;
+        if (ph == 0) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) low[k] = other_row(low[k]);
+        }
       }
     }
     if constexpr (SPA == PDF) {

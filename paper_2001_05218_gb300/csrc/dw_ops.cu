@@ -16,7 +16,9 @@ dw_status check_op(const dw_field* U, const dw_field* in, const dw_field* out) {
 }
 
 void apply_plan(Plan& P, const dw_field* U, const dw_field* in) {
+  // untuned: the FP64-class stencils run best in blocks of 64 sites (see the solver's plan)
   BlockShape shape{0, 0};
+  if (in->prec == DW_F64 || in->prec == DW_DF64) shape = BlockShape{64, 1};
   tune_lookup(tune_key(&U->lat, 1, in->nrhs, U->prec, U->compress12), &shape);
   make_plan(P, &U->lat, 1, in->nrhs, shape.T, shape.RB);
   P.pair = shape.pair;

@@ -83,7 +83,8 @@ struct CG {
   static constexpr int kLinkLo = S_LLO;
 
   // reliable update (gated by do_rel) and its finalizer
-  static void reliable(const Exec& E, int mode, RelCond rc = RelCond{0, 0}) {
+  // (EH: the plan of the high-precision stencils)
+  static void reliable(const Exec& E, const Exec& EH, int mode, RelCond rc = RelCond{0, 0}) {
     // even-odd systems: x_e += xl_e (xl_e = 0); t_o = H_oe x_e; r_e = bh - x_e + k^2 H_eo t_o
     // (MODE_HERM: the same with the Laplacian's K)
     auto eo_reliable = [&] {
@@ -91,8 +92,8 @@ struct CG {
       k_fold_x<L, A, H><<<E.grid(0), E.P.block, 0, E.st>>>(E.P.B, 0, E.ra(FIN_STORE0));
       // grid directions alternate: fold forwards, H_oe backwards, H_eo forwards
       // (the next stencil, z's first hop, walks backwards again)
-      hop<H, H, false, false, OP>(E.flipped(), 1, kLinkHi, InOne<H>{S_X}, EpiOut<H, C_ONE>{S_RT, G_REL});
-      hop<H, H, false, false, OP>(E, 0, kLinkHi, InOne<H>{S_RT}, EpiResidEO<L, H>{G_REL}, FIN_RELIABLE, rc);
+      hop<H, H, false, false, OP>(EH.flipped(), 1, kLinkHi, InOne<H>{S_X}, EpiOut<H, C_ONE>{S_RT, G_REL});
+      hop<H, H, false, false, OP>(EH, 0, kLinkHi, InOne<H>{S_RT}, EpiResidEO<L, H>{G_REL}, FIN_RELIABLE, rc);
     };
     if constexpr (OP == OP_LAPLACE) {
       eo_reliable();
@@ -101,14 +102,14 @@ struct CG {
     } else if (mode == MODE_FULL) {
       count_launch();
       k_fold_x<L, A, H><<<E.grid(2), E.P.block, 0, E.st>>>(E.P.B, 2, E.ra(FIN_STORE0));
-      hop<H, H, false, false, OP>(E, 2, kLinkHi, InOne<H>{S_X}, EpiResidFull<L, true, H>{G_REL, S_RT, S_X, S_B},
+      hop<H, H, false, false, OP>(EH, 2, kLinkHi, InOne<H>{S_X}, EpiResidFull<L, true, H>{G_REL, S_RT, S_X, S_B},
                               FIN_RELIABLE, rc);
     } else {
       count_launch();
       k_fold_x<L, A, H><<<E.grid(2), E.P.block, 0, E.st>>>(E.P.B, 2, E.ra(FIN_STORE0));
       // t = D x ; r = b - D^dag t
-      hop<H, H, false, false, OP>(E, 2, kLinkHi, InOne<H>{S_X}, EpiXpay<H, H, C_MK, false>{S_AUX0, S_X, G_REL});
-      hop<H, H, false, true, OP>(E, 2, kLinkHi, InOne<H>{S_AUX0}, EpiResidFull<L, true, H>{G_REL, S_RT, S_AUX0, S_B},
+      hop<H, H, false, false, OP>(EH, 2, kLinkHi, InOne<H>{S_X}, EpiXpay<H, H, C_MK, false>{S_AUX0, S_X, G_REL});
+      hop<H, H, false, true, OP>(EH, 2, kLinkHi, InOne<H>{S_AUX0}, EpiResidFull<L, true, H>{G_REL, S_RT, S_AUX0, S_B},
                              FIN_RELIABLE, rc);
     }
   }
@@ -148,9 +149,9 @@ struct CG {
   }
 
   static dw_status run(const SolveArgs& a);
-  static dw_status build_graph(const Exec& E, int mode, cudaGraphExec_t* exec, int* body_kernels,
+  static dw_status build_graph(const Exec& E, const Exec& EH, int mode, cudaGraphExec_t* exec, int* body_kernels,
                                int* rel_kernels);
-  static dw_status run_stepped(const Exec& E, int mode, int maxiter);
+  static dw_status run_stepped(const Exec& E, const Exec& EH, int mode, int maxiter);
 
   // The iterations in one kernel (k_cg_loop): even-odd Wilson systems in FP32 or
   // 16 bits with blocks of 32 sites, few enough columns and tiles for its sums.
@@ -209,8 +210,8 @@ dw_status CG<L, A, C12, H, OP>::launch_loop(const Exec& E, cudaGraphConditionalH
 // the loop is capped at maxiter + 2 passes, and every column also leaves the
 // loop through its own maxiter / timeout / breakdown checks.
 template <int L, int A, bool C12, int H, int OP>
-dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, int mode, cudaGraphExec_t* exec, int* body_kernels,
-                                        int* rel_kernels) {
+dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, const Exec& EH0, int mode, cudaGraphExec_t* exec,
+                                        int* body_kernels, int* rel_kernels) {
   static thread_local CaptureStreams cs;
   const int pm = eo_mode(mode) ? 0 : 2;
   cudaGraph_t g = nullptr;
@@ -281,7 +282,9 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, int mode, cudaGraphE
     c1 = pr.launches;
     DW_CUDA(cudaStreamBeginCaptureToGraph(cs.b, ip.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                           cudaStreamCaptureModeThreadLocal));
-    reliable(R, mode, one ? RelCond{(unsigned long long)hw, 2} : RelCond{0, 3});
+    Exec RH = EH0;
+    RH.st = cs.b;
+    reliable(R, RH, mode, one ? RelCond{(unsigned long long)hw, 2} : RelCond{0, 3});
     cudaGraph_t tmp;
     DW_CUDA(cudaStreamEndCapture(cs.b, &tmp));
     c2 = pr.launches;
@@ -317,7 +320,7 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, int mode, cudaGraphE
 // after every update so that no launch is made without work; used while the
 // launch profiler is active.
 template <int L, int A, bool C12, int H, int OP>
-dw_status CG<L, A, C12, H, OP>::run_stepped(const Exec& E, int mode, int maxiter) {
+dw_status CG<L, A, C12, H, OP>::run_stepped(const Exec& E, const Exec& EH, int mode, int maxiter) {
   static Flags* hf = nullptr;
   if (!hf) DW_CUDA(cudaMallocHost((void**)&hf, sizeof(Flags)));
   const int pm = eo_mode(mode) ? 0 : 2;
@@ -331,7 +334,7 @@ dw_status CG<L, A, C12, H, OP>::run_stepped(const Exec& E, int mode, int maxiter
     finish(E, pm, FIN_UPDATE);
     DW_CUDA(cudaMemcpyAsync(hf, E.rb.flags, sizeof(Flags), cudaMemcpyDeviceToHost, E.st));
     DW_CUDA(cudaStreamSynchronize(E.st));
-    if (hf->rel_pending > 0) reliable(E, mode);
+    if (hf->rel_pending > 0) reliable(E, EH, mode);
     if (hf->active == 0) continue;
     zstep(E, mode, FIN_BETA);
     count_launch();
@@ -394,6 +397,14 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
     }
     make_plan(F.P, lats, nrhs, shape.T, shape.RB);
     F.P.pair = shape.pair;
+    // High-precision stencils (two threads per site) run in blocks of 64 sites
+    // whatever suits the inner ones: a double-float 32^3x64 application takes
+    // 808 / 733 / 723 / 723 us with 256 / 128 / 64 / 32 sites per block, IEEE FP64 is
+    // the same from 128 down.
+    Exec& FH = fresh.EH;
+    if (OP == OP_WILSON) make_plan(FH.P, lats, nrhs, 64, 1);
+    else FH.P = F.P;
+    const int partials = F.P.partials > FH.P.partials ? F.P.partials : FH.P.partials;
     auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
     struct Piece { int slot, prec, npar; };
     std::vector<Piece> pieces;
@@ -421,11 +432,11 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
         total += al((size_t)nrhs * pc.npar * spin_bytes(pc.prec) * vh);
       }
     }
-    const size_t red_bytes = al(sizeof(DF) * F.P.partials) + al(sizeof(ColState) * F.P.ncols) + al(sizeof(Flags));
+    const size_t red_bytes = al(sizeof(DF) * partials) + al(sizeof(ColState) * F.P.ncols) + al(sizeof(Flags));
     DW_CUDA(device_alloc(&fresh.arena, total + red_bytes));
     char* rp = fresh.arena + total;
     F.rb.partial = reinterpret_cast<DF*>(rp);
-    rp += al(sizeof(DF) * F.P.partials);
+    rp += al(sizeof(DF) * partials);
     F.rb.cols = reinterpret_cast<ColState*>(rp);
     rp += al(sizeof(ColState) * F.P.ncols);
     F.rb.flags = reinterpret_cast<Flags*>(rp);
@@ -451,16 +462,18 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
           fresh.zero.push_back({S.f[S_RT].p + r * S.f[S_RT].rhs_stride + S.f[S_RT].par_stride,
                                 (size_t)spin_bytes(H) * S.vh});
     }
-    F.st = st;
-    dw_status gs = build_graph(F, mode, &fresh.exec, &fresh.body_k, &fresh.rel_k);
+    for (int i = 0; i < n; ++i) memcpy(FH.P.B.sd[i].f, F.P.B.sd[i].f, sizeof F.P.B.sd[i].f);
+    FH.rb = F.rb;
+    F.st = FH.st = st;
+    dw_status gs = build_graph(F, FH, mode, &fresh.exec, &fresh.body_k, &fresh.rel_k);
     if (gs != DW_OK) {
       cudaFree(fresh.arena);
       return gs;
     }
     ent = solve_cache_insert(std::move(fresh));
   }
-  Exec E = ent->E;
-  E.st = st;
+  Exec E = ent->E, EH = ent->EH;
+  E.st = EH.st = st;
 
   // ---- column state
   std::vector<ColState> hc(E.P.ncols);
@@ -505,7 +518,7 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
   for (auto& z : ent->zero) DW_CUDA(cudaMemsetAsync(z.first, 0, z.second, st));
   if (eo) {
     // bh = b_e + kappa H_eo b_o
-    hop<H, H, false, false, OP>(E, 0, kLinkHi, InOne<H>{S_B}, EpiXpay<H, H, C_PK, false>{S_BH, S_B, G_ALL});
+    hop<H, H, false, false, OP>(EH, 0, kLinkHi, InOne<H>{S_B}, EpiXpay<H, H, C_PK, false>{S_BH, S_B, G_ALL});
   }
   // zero guess: r = source (bh or b); otherwise r = source - A x, recomputed
   count_launch();
@@ -518,9 +531,9 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
     if (!hf0) DW_CUDA(cudaMallocHost((void**)&hf0, sizeof(Flags)));
     DW_CUDA(cudaMemcpyAsync(hf0, E.rb.flags, sizeof(Flags), cudaMemcpyDeviceToHost, st));
     DW_CUDA(cudaStreamSynchronize(st));
-    if (hf0->rel_pending > 0) reliable(E, mode);
+    if (hf0->rel_pending > 0) reliable(E, EH, mode);
   } else {
-    reliable(E, mode);
+    reliable(E, EH, mode);
   }
   zstep(E, mode, FIN_GAMMA0);  // z, gamma
   count_launch();
@@ -533,7 +546,7 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
   if (graph) {
     DW_CUDA(cudaGraphLaunch(ent->exec, st));
   } else {
-    DW_TRY(run_stepped(E, mode, a.p.maxiter));
+    DW_TRY(run_stepped(E, EH, mode, a.p.maxiter));
   }
 
   // ---- finish: odd sites, then the IEEE FP64 residual from the caller's fields
@@ -551,14 +564,14 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
   k_zero_zsrc<P64><<<E.grid(2), E.P.block, 0, st>>>(E.P.B, 2, S_XU, E.ra(FIN_STORE0));  // zero source: x = 0
   const int rt64 = H == P64 ? S_RT : S_AUX1;  // FP64 full temporary (verify_normal)
   if (mode != MODE_NORMAL) {
-    hop<P64, P64, false, false, OP>(E, 2, S_LF64, InOne<P64>{S_XU},
+    hop<P64, P64, false, false, OP>(EH, 2, S_LF64, InOne<P64>{S_XU},
                                 EpiResidFull<L, false, P64>{G_ALL, a.p.verify_normal ? rt64 : -1, S_XU, S_BU},
                                 FIN_STORE0);
     if constexpr (OP == OP_WILSON) {
       if (a.p.verify_normal) {
-        hop<P64, P64, false, true, OP>(E, 2, S_LF64, InOne<P64>{rt64}, EpiXpay<P64, P64, C_MK, true>{-1, rt64, G_ALL},
+        hop<P64, P64, false, true, OP>(EH, 2, S_LF64, InOne<P64>{rt64}, EpiXpay<P64, P64, C_MK, true>{-1, rt64, G_ALL},
                                        FIN_STORE1);
-        hop<P64, P64, false, true, OP>(E, 2, S_LF64, InOne<P64>{S_BU}, EpiXpay<P64, P64, C_MK, true>{-1, S_BU, G_ALL},
+        hop<P64, P64, false, true, OP>(EH, 2, S_LF64, InOne<P64>{S_BU}, EpiXpay<P64, P64, C_MK, true>{-1, S_BU, G_ALL},
                                        FIN_STORE2);
       }
     }
@@ -566,9 +579,9 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
     if constexpr (OP == OP_WILSON) {
       // |b - D^dag D x|^2 in FP64: t = D x into the FP64 temporary, then b - D^dag t
       const int t64 = H == P64 ? S_AUX0 : S_AUX1;
-      hop<P64, P64, false, false, OP>(E, 2, S_LF64, InOne<P64>{S_XU},
+      hop<P64, P64, false, false, OP>(EH, 2, S_LF64, InOne<P64>{S_XU},
                                       EpiXpay<P64, P64, C_MK, false>{t64, S_XU, G_ALL});
-      hop<P64, P64, false, true, OP>(E, 2, S_LF64, InOne<P64>{t64}, EpiResidFull<L, false, P64>{G_ALL, -1, t64, S_BU},
+      hop<P64, P64, false, true, OP>(EH, 2, S_LF64, InOne<P64>{t64}, EpiResidFull<L, false, P64>{G_ALL, -1, t64, S_BU},
                                      FIN_STORE0);
     }
   }
