@@ -54,21 +54,16 @@ struct Exec {
   Plan P;
   RedBuf rb;
   cudaStream_t st = nullptr;
-  // 1: the launches walk their grid from its end (Batch::rev).  Consecutive
+  // Batch::rev = 1: the launches walk their grid from its end.  Consecutive
   // kernels of a CG iteration alternate directions, so that each starts on
   // the sites (links, neighbour spinors, the vector just written) that its
   // predecessor touched last and that are still in L2 (measured on GB300:
   // FP16 stencils 1.8% and the 32^3x64 solve 0.9% faster; results unchanged,
   // since the block partials stay indexed by tile).
-  int rev = 0;
-  Batch batch() const {
-    Batch b = P.B;
-    b.rev = rev;
-    return b;
-  }
+  const Batch& batch() const { return P.B; }
   Exec flipped() const {
     Exec e = *this;
-    e.rev = 1 - rev;
+    e.P.B.rev = 1 - P.B.rev;
     return e;
   }
   RedArgs ra(int fin) const {
@@ -137,6 +132,20 @@ inline void finish(const Exec& E, int par_mode, int fin, RelCond rel = RelCond{0
   }
 }
 
+// kernel<<<grid, block, smem, st>>>(args...) without the copies of the launch
+// syntax: the 4.6 KB plan is read in place (its copies pushed the caller's data
+// out of the L1 cache on every operator application).
+template <class T>
+struct exact {
+  using type = T;
+};
+template <class... P>
+inline void launch(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st,
+                   const typename exact<P>::type&... args) {
+  void* p[] = {const_cast<void*>(static_cast<const void*>(&args))...};
+  cudaLaunchKernel(reinterpret_cast<const void*>(kernel), grid, dim3(block), p, smem, st);
+}
+
 // More than 48 KiB of dynamic shared memory for a kernel on the current device.
 template <class K>
 inline void allow_shared(K* kernel, size_t bytes) {
@@ -161,15 +170,16 @@ inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int 
   if constexpr (kRows) {
     const size_t smem = SPA == PDF ? (size_t)E.P.block.x / 16 * RowRing<C12>::kBytes : 0;
     if (smem > 48 * 1024) allow_shared(k_hop_rows<SPA, C12, DAG, Epi>, smem);
-    k_hop_rows<SPA, C12, DAG, Epi><<<E.grid(par_mode), 2 * E.P.block.x, smem, E.st>>>(
-        E.batch(), par_mode, link_slot, in.slot, epi, E.ra(fin));
+    launch(k_hop_rows<SPA, C12, DAG, Epi>, E.grid(par_mode), 2 * E.P.block.x, smem, E.st, E.batch(), par_mode, link_slot,
+           in.slot, epi, E.ra(fin));
     launched = true;
   }
   if constexpr ((SPA == P16 || SPA == PB16) && LP == SPA && OP == OP_WILSON && std::is_same<In, InOne<SPA>>::value) {
     if (E.P.pair == 1 && E.P.nrhs >= 2) {  // two right-hand sides per thread, each link loaded once for both
       const unsigned npar = par_mode == 2 ? 2u : 1u;
       const dim3 g(npar * E.P.B.ntot * ((E.P.nrhs + 2 * E.P.B.RB - 1) / (2 * E.P.B.RB)));
-      k_hop_pair<SPA, C12, DAG, Epi><<<g, E.P.block, 0, E.st>>>(E.batch(), par_mode, link_slot, in.slot, epi, E.ra(fin));
+      launch(k_hop_pair<SPA, C12, DAG, Epi>, g, E.P.block.x, 0, E.st, E.batch(), par_mode, link_slot, in.slot, epi,
+             E.ra(fin));
       launched = true;
     }
   }
@@ -177,14 +187,15 @@ inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int 
   if constexpr (SPA != P64 && SPA != PDF && LP == SPA && OP == OP_WILSON && std::is_same<In, InOne<SPA>>::value) {
     if (E.P.pair == 2) {
       const unsigned n = E.P.block.x;
-      k_hop_split<SPA, LP, C12, DAG, In, Epi><<<E.grid(par_mode), 4 * n, n / 32 * (3 * 24 * 32 * sizeof(float)), E.st>>>(
-          E.batch(), par_mode, link_slot, in, epi, E.ra(fin));
+      launch(k_hop_split<SPA, LP, C12, DAG, In, Epi>, E.grid(par_mode), 4 * n, n / 32 * (3 * 24 * 32 * sizeof(float)), E.st,
+             E.batch(), par_mode, link_slot, in, epi, E.ra(fin));
       launched = true;
     }
   }
   if constexpr (!kRows) {
-    if (!launched) k_hop<SPA, LP, C12, DAG, In, Epi, OP><<<E.grid(par_mode), E.P.block, 0, E.st>>>(E.batch(), par_mode, link_slot, in,
-                                                                                    epi, E.ra(fin));
+    if (!launched)
+      launch(k_hop<SPA, LP, C12, DAG, In, Epi, OP>, E.grid(par_mode), E.P.block.x, 0, E.st, E.batch(), par_mode, link_slot, in,
+             epi, E.ra(fin));
   }
   if (pr.timing) {
     cudaEventRecord(eb, E.st);

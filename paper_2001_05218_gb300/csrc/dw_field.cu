@@ -136,7 +136,7 @@ void default_block_shape(int nrhs, int* T, int* RB) {
 }
 
 void make_plan(Plan& P, const dw_lattice* lats, int n, int nrhs, int T, int RB) {
-  memset(&P.B, 0, sizeof P.B);
+  P.B.rev = 0;  // descriptors past the last system stay as they are: no kernel reads them
   P.pair = 0;
   P.nsys = n;
   P.nrhs = nrhs;

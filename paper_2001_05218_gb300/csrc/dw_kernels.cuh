@@ -602,9 +602,14 @@ struct EpiXpayDot {
   template <typename R>
   __device__ __forceinline__ Packed prepare(const SysDesc& S, int par, int r, int s, Cx<R> (&acc)[12],
                                             typename RedT<R>::type& nrm) const {
-    using RO = typename Spin<SPO>::R;
     Cx<typename Spin<SPX>::R> xv[12];
     Spin<SPX>::load(slot_ptr(S, slot_x, r, par), S.vh, s, xv);
+    return form(S, acc, xv, nrm);
+  }
+  template <typename R>
+  __device__ __forceinline__ Packed form(const SysDesc& S, Cx<R> (&acc)[12], const Cx<typename Spin<SPX>::R> (&xv)[12],
+                                         typename RedT<R>::type& nrm) const {
+    using RO = typename Spin<SPO>::R;
     const R c = coef<COEF, R>(S);
     Cx<RO> o[12];
     R n = (R)0;

@@ -39,7 +39,6 @@
 
 namespace dw {
 
-enum Mode { MODE_EO = 0, MODE_FULL = 1, MODE_NORMAL = 2, MODE_HERM = 3 };
 // modes whose CG vectors live on the even sites only
 inline bool eo_mode(int mode) { return mode == MODE_EO || mode == MODE_HERM; }
 // plain CG: the search direction is built from r itself
@@ -51,9 +50,10 @@ inline long long parity_work(const std::vector<dw_lattice>& lats, int nrhs) {
   for (auto& l : lats) sites += vh_of(l) * nrhs;
   return sites;
 }
-// Small systems run in blocks of 32 sites: up to kSplitSites with four threads
-// per site (k_hop_split), and even-odd systems up to kLoopSites with all
-// iterations in one kernel (k_cg_loop).
+// Small systems run in blocks of 32 sites: Wilson systems up to kSplitSites with
+// four threads per site (k_hop_split), and systems up to kLoopSites (both
+// parities counted where the vectors have both) with all iterations in one
+// kernel (k_cg_loop).
 constexpr long long kSplitSites = 16384, kLoopSites = 65536;
 
 struct SolveArgs {
@@ -153,16 +153,16 @@ struct CG {
                                int* rel_kernels);
   static dw_status run_stepped(const Exec& E, const Exec& EH, int mode, int maxiter);
 
-  // The iterations in one kernel (k_cg_loop): even-odd Wilson systems in FP32 or
-  // 16 bits with blocks of 32 sites, few enough columns and tiles for its sums.
-  static constexpr bool kLoop = OP == OP_WILSON && L != P64 && L != PDF;
+  // The iterations in one kernel (k_cg_loop): FP32 and 16-bit systems with blocks
+  // of 32 sites, few enough columns and tiles for its sums.
+  static constexpr bool kLoop = L != P64 && L != PDF;
   static bool loop_fits(const Plan& P, int mode) {
-    if (!kLoop || mode != MODE_EO || P.B.T != 32 || P.B.RB != 1 || P.ncols > kLoopCols) return false;
+    if (!kLoop || mode == MODE_FULL || P.B.T != 32 || P.B.RB != 1 || P.ncols > kLoopCols) return false;
     for (int i = 0; i < P.nsys; ++i)
-      if (P.B.sd[i].tpp > kLoopPartials) return false;
+      if (P.B.sd[i].tpp * (eo_mode(mode) ? 1 : 2) > kLoopPartials) return false;
     return true;
   }
-  static dw_status launch_loop(const Exec& E, cudaGraphConditionalHandle rel, cudaGraphConditionalHandle loop);
+  static dw_status launch_loop(const Exec& E, int mode, cudaGraphConditionalHandle rel, cudaGraphConditionalHandle loop);
 };
 
 struct CaptureStreams {
@@ -174,7 +174,7 @@ struct CaptureStreams {
 };
 
 template <int L, int A, bool C12, int H, int OP>
-dw_status CG<L, A, C12, H, OP>::launch_loop(const Exec& E, cudaGraphConditionalHandle rel,
+dw_status CG<L, A, C12, H, OP>::launch_loop(const Exec& E, int mode, cudaGraphConditionalHandle rel,
                                             cudaGraphConditionalHandle loop) {
   if constexpr (kLoop) {
     // a block takes at least four 32-site items, and one block runs per SM: more
@@ -182,7 +182,7 @@ dw_status CG<L, A, C12, H, OP>::launch_loop(const Exec& E, cudaGraphConditionalH
     int dev = 0, sms = 0;
     DW_CUDA(cudaGetDevice(&dev));
     DW_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int items = E.P.B.ntot * E.P.nrhs;
+    const int items = E.P.B.ntot * E.P.nrhs * (eo_mode(mode) ? 1 : 2);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeCooperative;
     at[0].val.cooperative = 1;
@@ -193,13 +193,15 @@ dw_status CG<L, A, C12, H, OP>::launch_loop(const Exec& E, cudaGraphConditionalH
     lc.attrs = at;
     lc.numAttrs = 1;
     count_launch();
-    const RedArgs ra = E.ra(FIN_STORE0);
-    if (E.P.pair == 2)
-      DW_CUDA(cudaLaunchKernelEx(&lc, k_cg_loop<L, A, C12, true>, E.P.B, ra, (unsigned long long)rel,
-                                 (unsigned long long)loop));
-    else
-      DW_CUDA(cudaLaunchKernelEx(&lc, k_cg_loop<L, A, C12, false>, E.P.B, ra, (unsigned long long)rel,
-                                 (unsigned long long)loop));
+    void (*k)(Batch, RedArgs, unsigned long long, unsigned long long) = nullptr;
+    if constexpr (OP == OP_LAPLACE) {
+      k = k_cg_loop<L, A, C12, false, MODE_HERM>;
+    } else if (mode == MODE_NORMAL) {
+      k = E.P.pair == 2 ? k_cg_loop<L, A, C12, true, MODE_NORMAL> : k_cg_loop<L, A, C12, false, MODE_NORMAL>;
+    } else {
+      k = E.P.pair == 2 ? k_cg_loop<L, A, C12, true, MODE_EO> : k_cg_loop<L, A, C12, false, MODE_EO>;
+    }
+    DW_CUDA(cudaLaunchKernelEx(&lc, k, E.P.B, E.ra(FIN_STORE0), (unsigned long long)rel, (unsigned long long)loop));
   }
   return DW_OK;
 }
@@ -242,7 +244,7 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, const Exec& EH0, int
   DW_CUDA(cudaStreamBeginCaptureToGraph(cs.a, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
   const bool one = loop_fits(E.P, mode);
   if (one) {
-    DW_TRY(launch_loop(E, hr, hw));
+    DW_TRY(launch_loop(E, mode, hr, hw));
   } else {
     // A pass of the while node and the test of the if node cost about 4 us each
     // (empty kernels in such a graph: 4.5 us per pass, 8.0 with the if node, 0.6
@@ -390,10 +392,10 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
     Exec& F = fresh.E;
     BlockShape shape{a.p.tile, a.p.tile > 0 ? 1 : 0};
     if (a.p.tile <= 0) shape = tune_inner_shape<L, C12>(lats, nrhs, lo_links, st);
-    if (a.p.tile <= 0 && OP == OP_WILSON && L != P64 && L != PDF) {
+    if (a.p.tile <= 0 && L != P64 && L != PDF) {
       const long long work = parity_work(lats, nrhs);
-      if (work <= kSplitSites) shape = BlockShape{32, 1, 2};
-      else if (mode == MODE_EO && work <= kLoopSites && n * nrhs <= kLoopCols) shape = BlockShape{32, 1, 0};
+      if (OP == OP_WILSON && work <= kSplitSites) shape = BlockShape{32, 1, 2};
+      else if (mode != MODE_FULL && work * fpar <= kLoopSites && n * nrhs <= kLoopCols) shape = BlockShape{32, 1, 0};
     }
     make_plan(F.P, lats, nrhs, shape.T, shape.RB);
     F.P.pair = shape.pair;
@@ -404,7 +406,9 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
     Exec& FH = fresh.EH;
     if (OP == OP_WILSON) make_plan(FH.P, lats, nrhs, 64, 1);
     else FH.P = F.P;
-    const int partials = F.P.partials > FH.P.partials ? F.P.partials : FH.P.partials;
+    // (k_cg_loop keeps two sets of partials; with one parity the plan has room for both)
+    const int inner = (eo ? 1 : 2) * F.P.partials;
+    const int partials = inner > FH.P.partials ? inner : FH.P.partials;
     auto al = [](size_t v) { return (v + 255) & ~(size_t)255; };
     struct Piece { int slot, prec, npar; };
     std::vector<Piece> pieces;
