@@ -1603,20 +1603,64 @@ __global__ void __launch_bounds__(256) k_norm(const __grid_constant__ Batch B, i
   DW_BLOCK_REDUCE(nrm)
 }
 
+// dst = convert(src) and |src|^2 -> finalizer ra.fin, in one pass over src (gate: all)
+template <int SPD, int SPS>
+__global__ void __launch_bounds__(256) k_convert_norm(const __grid_constant__ Batch B, int par_mode, int slot_dst,
+                                                      int slot_src, RedArgs ra) {
+  DW_BLOCK_PROLOGUE(G_ALL)
+  using RS = typename Spin<SPS>::R;
+  typename RedT<RS>::type nrm = red_zero(typename RedT<RS>::type());
+  if (valid) {
+    Cx<RS> v[12];
+    Cx<typename Spin<SPD>::R> o[12];
+    Spin<SPS>::load(slot_ptr(S, slot_src, r, par), S.vh, s, v);
+    RS n = (RS)0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) n = fma(v[k].re, v[k].re, fma(v[k].im, v[k].im, n));
+    nrm = to_red(n);
+    convert12(v, o);
+    Spin<SPD>::store(slot_wptr(S, slot_dst, r, par), S.vh, s, o);
+  }
+  DW_BLOCK_REDUCE(nrm)
+}
+
 // Odd-site reconstruction x_o = b_o + kappa t_o, t_o = H_oe x_e as left in the
 // odd half of S_RT by the last reliable update, in the high precision SPH.
+template <int SPH, typename R>
+__device__ __forceinline__ void recon_odd(const SysDesc& S, int r, int s, Cx<R> (&xv)[12]) {
+  Cx<R> bv[12], tv[12];
+  Spin<SPH>::load(slot_ptr(S, S_B, r, 1), S.vh, s, bv);
+  Spin<SPH>::load(slot_ptr(S, S_RT, r, 1), S.vh, s, tv);
+  const R k = coef<C_PK, R>(S);
+#pragma unroll
+  for (int j = 0; j < 12; ++j) xv[j] = cx(fma(k, tv[j].re, bv[j].re), fma(k, tv[j].im, bv[j].im));
+}
 template <int SPH>
 __global__ void __launch_bounds__(256) k_recon_odd(const __grid_constant__ Batch B, int par_mode, RedArgs ra) {
   DW_BLOCK_PROLOGUE(G_ALL)
   if (valid) {
-    using RH = typename Spin<SPH>::R;
-    Cx<RH> bv[12], tv[12], xv[12];
-    Spin<SPH>::load(slot_ptr(S, S_B, r, par), S.vh, s, bv);
-    Spin<SPH>::load(slot_ptr(S, S_RT, r, par), S.vh, s, tv);
-    const RH k = coef<C_PK, RH>(S);
-#pragma unroll
-    for (int j = 0; j < 12; ++j) xv[j] = cx(fma(k, tv[j].re, bv[j].re), fma(k, tv[j].im, bv[j].im));
+    Cx<typename Spin<SPH>::R> xv[12];
+    recon_odd<SPH>(S, r, s, xv);
     Spin<SPH>::store(slot_wptr(S, S_X, r, par), S.vh, s, xv);
+  }
+}
+
+// The caller's solution (FP64) from the accumulator in SPH: S_XU <- S_X, on odd
+// sites of an even-odd system (recon) the reconstruction, 0 for a zero source.
+// One pass instead of reconstruction, conversion and zeroing (32^3x64: 228 us in
+// three kernels, the odd sites written and read once more in between).
+template <int SPH>
+__global__ void __launch_bounds__(256) k_solution(const __grid_constant__ Batch B, int par_mode, int recon, RedArgs ra) {
+  DW_BLOCK_PROLOGUE(G_ALL)
+  if (valid) {
+    Cx<typename Spin<SPH>::R> xv[12];
+    Cx<double> o[12];
+    if (recon && par == 1) recon_odd<SPH>(S, r, s, xv);
+    else Spin<SPH>::load(slot_ptr(S, S_X, r, par), S.vh, s, xv);
+    const bool zero = ra.cols[S.col0 + r].zsrc != 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) o[k] = zero ? cx(0.0, 0.0) : cx((double)xv[k].re, (double)xv[k].im);
+    Spin<P64>::store(slot_wptr(S, S_XU, r, par), S.vh, s, o);
   }
 }
 
@@ -1629,20 +1673,6 @@ __global__ void __launch_bounds__(256) k_zero_zsrc(const __grid_constant__ Batch
 #pragma unroll
     for (int k = 0; k < 12; ++k) z[k] = cx((typename Spin<SP>::R)0, (typename Spin<SP>::R)0);
     Spin<SP>::store(slot_wptr(S, slot, r, par), S.vh, s, z);
-  }
-}
-
-// dst = convert(src), over the launched parities (gate: all)
-template <int SPD, int SPS>
-__global__ void __launch_bounds__(256) k_convert(const __grid_constant__ Batch B, int par_mode, int slot_dst, int slot_src,
-                                                 RedArgs ra) {
-  DW_BLOCK_PROLOGUE(G_ALL)
-  if (valid) {
-    Cx<typename Spin<SPS>::R> v[12];
-    Cx<typename Spin<SPD>::R> o[12];
-    Spin<SPS>::load(slot_ptr(S, slot_src, r, par), S.vh, s, v);
-    convert12(v, o);
-    Spin<SPD>::store(slot_wptr(S, slot_dst, r, par), S.vh, s, o);
   }
 }
 

@@ -53,7 +53,9 @@ inline long long parity_work(const std::vector<dw_lattice>& lats, int nrhs) {
 // Small systems run in blocks of 32 sites: Wilson systems up to kSplitSites with
 // four threads per site (k_hop_split), and systems up to kLoopSites (both
 // parities counted where the vectors have both) with all iterations in one
-// kernel (k_cg_loop).
+// kernel (k_cg_loop).  Beyond that its 16 warps per SM lose to the separate
+// kernels: solves with 65536 / 81920 / 131072 sites of a parity, FP16, one kernel
+// 3.16 / 4.54 / 5.25 ms, separate 3.67 / 3.84 / 4.93 ms.
 constexpr long long kSplitSites = 16384, kLoopSites = 65536;
 
 struct SolveArgs {
@@ -511,13 +513,18 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
   }
 
   // ---- set-up
-  norm<P64>(E, 2, S_BU, FIN_BNORM);
-  norm<P64>(E, eo ? 0 : 2, S_XU, FIN_XNORM);
-  if (H != P64) {
+  if (H == P64) {
+    norm<P64>(E, 2, S_BU, FIN_BNORM);
+    norm<P64>(E, eo ? 0 : 2, S_XU, FIN_XNORM);
+  } else {
+    // high-precision copies and norms in one pass each (at 32^3x64 two norms and
+    // two conversions took 393 us); even-odd systems read x on even sites only
     count_launch();
-    k_convert<H, P64><<<E.grid(2), E.P.block, 0, st>>>(E.P.B, 2, S_B, S_BU, E.ra(FIN_STORE0));
+    k_convert_norm<H, P64><<<E.grid(2), E.P.block, 0, st>>>(E.P.B, 2, S_B, S_BU, E.ra(FIN_STORE0));
+    finish(E, 2, FIN_BNORM);
     count_launch();
-    k_convert<H, P64><<<E.grid(2), E.P.block, 0, st>>>(E.P.B, 2, S_X, S_XU, E.ra(FIN_STORE0));
+    k_convert_norm<H, P64><<<E.grid(eo ? 0 : 2), E.P.block, 0, st>>>(E.P.B, eo ? 0 : 2, S_X, S_XU, E.ra(FIN_STORE0));
+    finish(E, eo ? 0 : 2, FIN_XNORM);
   }
   for (auto& z : ent->zero) DW_CUDA(cudaMemsetAsync(z.first, 0, z.second, st));
   if (eo) {
@@ -554,18 +561,20 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
   }
 
   // ---- finish: odd sites, then the IEEE FP64 residual from the caller's fields
-  if (eo) {
-    // x_o = b_o + kappa H_oe x_e, with H_oe x_e (the first hop of the column's
-    // last reliable update, taken of its final x_e) read from the odd half of S_RT
-    count_launch();
-    k_recon_odd<H><<<E.grid(1), E.P.block, 0, st>>>(E.P.B, 1, E.ra(FIN_STORE0));
-  }
+  // (even-odd: x_o = b_o + kappa H_oe x_e, with H_oe x_e, the first hop of the
+  // column's last reliable update, taken of its final x_e, read from the odd half
+  // of S_RT); a zero source has the solution 0
   if (H != P64) {
     count_launch();
-    k_convert<P64, H><<<E.grid(2), E.P.block, 0, st>>>(E.P.B, 2, S_XU, S_X, E.ra(FIN_STORE0));
+    k_solution<H><<<E.grid(2), E.P.block, 0, st>>>(E.P.B, 2, eo ? 1 : 0, E.ra(FIN_STORE0));
+  } else {
+    if (eo) {
+      count_launch();
+      k_recon_odd<H><<<E.grid(1), E.P.block, 0, st>>>(E.P.B, 1, E.ra(FIN_STORE0));
+    }
+    count_launch();
+    k_zero_zsrc<P64><<<E.grid(2), E.P.block, 0, st>>>(E.P.B, 2, S_XU, E.ra(FIN_STORE0));
   }
-  count_launch();
-  k_zero_zsrc<P64><<<E.grid(2), E.P.block, 0, st>>>(E.P.B, 2, S_XU, E.ra(FIN_STORE0));  // zero source: x = 0
   const int rt64 = H == P64 ? S_RT : S_AUX1;  // FP64 full temporary (verify_normal)
   if (mode != MODE_NORMAL) {
     hop<P64, P64, false, false, OP>(EH, 2, S_LF64, InOne<P64>{S_XU},
