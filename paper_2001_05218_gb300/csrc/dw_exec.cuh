@@ -163,14 +163,13 @@ inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int 
     eb = pr.event();
     cudaEventRecord(ea, E.st);
   }
-  // FP64-class Wilson stencils: two threads per site
-  constexpr bool kRows =
-      (SPA == P64 || SPA == PDF) && LP == SPA && OP == OP_WILSON && std::is_same<In, InOne<SPA>>::value;
+  // FP64-class stencils: two threads per site
+  constexpr bool kRows = (SPA == P64 || SPA == PDF) && LP == SPA && std::is_same<In, InOne<SPA>>::value;
   bool launched = false;
   if constexpr (kRows) {
     const size_t smem = SPA == PDF ? (size_t)E.P.block.x / 16 * RowRing<C12>::kBytes : 0;
-    if (smem > 48 * 1024) allow_shared(k_hop_rows<SPA, C12, DAG, Epi>, smem);
-    launch(k_hop_rows<SPA, C12, DAG, Epi>, E.grid(par_mode), 2 * E.P.block.x, smem, E.st, E.batch(), par_mode, link_slot,
+    if (smem > 48 * 1024) allow_shared(k_hop_rows<SPA, C12, DAG, Epi, OP>, smem);
+    launch(k_hop_rows<SPA, C12, DAG, Epi, OP>, E.grid(par_mode), 2 * E.P.block.x, smem, E.st, E.batch(), par_mode, link_slot,
            in.slot, epi, E.ra(fin));
     launched = true;
   }

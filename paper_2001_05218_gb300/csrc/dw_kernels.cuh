@@ -596,8 +596,26 @@ struct EpiXpayDot {
     Spin<SPO>::store_packed(slot_wptr(S, slot_out, r, par), S.vh, s, o);
   }
   template <typename R>
-  __device__ __forceinline__ void write(const SysDesc& S, int par, int r, int s, Cx<R> (&acc)[12], double& nrm) const {
-    commit(S, par, r, s, prepare(S, par, r, s, acc, nrm));
+  __device__ __forceinline__ void write_rows(const SysDesc& S, int par, int r, int s, int row, Cx<R> (&a)[3],
+                                             Cx<R> (&b)[3], typename RedT<R>::type& nrm, bool ok) const {
+    const char* xp = slot_ptr(S, slot_x, r, par);
+    const R c = coef<COEF, R>(S);
+    R n = (R)0;
+    Cx<R> x[3];
+    Spin<SPX>::load_spin(xp, S.vh, s, row, x);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      a[k] = cx(fma(c, a[k].re, x[k].re), fma(c, a[k].im, x[k].im));
+      n = fma(x[k].re, a[k].re, fma(x[k].im, a[k].im, n));
+    }
+    Spin<SPX>::load_spin(xp, S.vh, s, 2 + row, x);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      b[k] = cx(fma(c, b[k].re, x[k].re), fma(c, b[k].im, x[k].im));
+      n = fma(x[k].re, b[k].re, fma(x[k].im, b[k].im, n));
+    }
+    nrm = to_red(n);
+    store_rows<SPO>(slot_wptr(S, slot_out, r, par), S.vh, s, row, a, b, ok);
   }
   template <typename R>
   __device__ __forceinline__ Packed prepare(const SysDesc& S, int par, int r, int s, Cx<R> (&acc)[12],
@@ -787,11 +805,8 @@ template <int SPA, int LP, bool C12, class In, typename R>
 __device__ __forceinline__ void laplace_dirs(const SysDesc& S, const In& in, const Coord& c, int s, int r, int pin,
                                              const char* ulink_own, const char* ulink_nb, long long mu_stride,
                                              Cx<R> (&acc)[12]) {
-  // FP32 and 16-bit: all eight directions unrolled (compile-time neighbour
-  // arithmetic); double-float and FP64 keep one copy of the loop body, whose
-  // unrolled form would not fit the instruction cache
-  constexpr int kUnroll = (SPA == PDF || SPA == P64) ? 1 : 8;
-#pragma unroll kUnroll
+  // all eight directions unrolled (compile-time neighbour arithmetic)
+#pragma unroll
   for (int d = 0; d < 8; ++d) {
     const int mu = d >> 1;
     const bool fwd = (d & 1) == 0;
@@ -846,17 +861,10 @@ __device__ __forceinline__ void laplace_dirs(const SysDesc& S, const In& in, con
         su3_mul<true>(u, h0, g0);
         su3_mul<true>(u, h1, g1);
       }
-      // double-float: sums left unnormalised, renormalised once after the
-      // eight directions (as the Wilson stencil's accumulation)
 #pragma unroll
       for (int k = 0; k < 6; ++k) {
-        if constexpr (std::is_same<R, DF>::value) {
-          acc[k] = cadd_lazy(acc[k], g0[k]);
-          acc[6 + k] = cadd_lazy(acc[6 + k], g1[k]);
-        } else {
-          acc[k] = acc[k] + g0[k];
-          acc[6 + k] = acc[6 + k] + g1[k];
-        }
+        acc[k] = acc[k] + g0[k];
+        acc[6 + k] = acc[6 + k] + g1[k];
       }
     }
   }
@@ -914,7 +922,7 @@ __device__ __forceinline__ void hop_mu(const SysDesc& S, const In& in, const Coo
 //   FP32, 18 reals   1: 284.5   2: 252.9   3: 306 (spills)
 //   FP32, 12 reals   1: 224.0   2: 211.2   3: 224
 //   I16, 12 reals    1: 181.8   2: 182.0   3: 179.4
-// Double-float (the Laplacian; the Wilson form has its own kernel): 2.
+// (FP64-class storage has its own kernel, k_hop_rows.)
 #ifndef DW_HOP16_MINB
 #define DW_HOP16_MINB 4
 #endif
@@ -927,7 +935,6 @@ __device__ __forceinline__ void hop_mu(const SysDesc& S, const In& in, const Coo
 template <int SPA>
 struct HopOccupancy {
   static constexpr int kMinBlocks = (SPA == P16 || SPA == PB16) ? DW_HOP16_MINB
-                                    : SPA == PDF                ? 2
                                     : SPA == P32                ? DW_HOP32_MINB
                                     : SPA == PI16               ? DW_HOPI16_MINB
                                                                 : 1;
@@ -954,10 +961,6 @@ __global__ void __launch_bounds__(256, HopOccupancy<SPA>::kMinBlocks)
 
       if constexpr (OP == OP_LAPLACE) {
         laplace_dirs<SPA, LP, C12>(S, in, c, s, r, pin, ulink_own, ulink_nb, mu_stride, acc);
-        if constexpr (SPA == PDF) {
-#pragma unroll
-          for (int k = 0; k < 12; ++k) acc[k] = cx(renorm(acc[k].re), renorm(acc[k].im));
-        }
       } else {
         hop_mu<0, SPA, LP, C12, SF>(S, in, c, s, r, pin, ulink_own, ulink_nb, mu_stride, acc);
         hop_mu<1, SPA, LP, C12, SF>(S, in, c, s, r, pin, ulink_own, ulink_nb, mu_stride, acc);
@@ -1216,12 +1219,54 @@ struct RowRing {
     }
   }
 };
+// The Laplacian's directions: both spins of the thread times U (or U^dag).
+template <bool C12, bool ADJ>
+__device__ __forceinline__ void lap_direction(const char* stage, int row, uint32_t bm, Cx<DF> (&up)[3], Cx<DF> (&low)[3]) {
+  using Ring = RowRing<C12>;
+  Cx<DF> h[6], g[6], u[9];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const Cx<DF> w = Ring::word(stage, k < 3 ? 3 * row + k : 3 * (2 + row) + k - 3);
+    h[k] = cx(flip(w.re, bm), flip(w.im, bm));
+  }
+#pragma unroll
+  for (int k = 0; k < Ring::kChunks - 12; ++k) u[k] = Ring::word(stage, 12 + k);
+  if (C12) rebuild_row2(u);
+  su3_mul<ADJ>(u, h, g);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    up[a] = row_add(up[a], g[a]);
+    low[a] = row_add(low[a], g[3 + a]);
+  }
+}
+// IEEE FP64: the products chained onto the sums, no additions of their own (1152
+// instead of 1344 FP64 operations per site).
+template <bool C12, bool ADJ>
+__device__ __forceinline__ void lap_direction(const SysDesc& S, const char* in, const char* lb, int n, int li, int row,
+                                              uint32_t bm, Cx<double> (&up)[3], Cx<double> (&low)[3]) {
+  Cx<double> a[3], b[3], u[9];
+  Spin<P64>::load_spin(in, S.vh, n, row, a);
+  Spin<P64>::load_spin(in, S.vh, n, 2 + row, b);
+  Link<P64, C12>::load(lb, S.vh, li, u);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    a[k] = cx(flip(a[k].re, bm), flip(a[k].im, bm));
+    b[k] = cx(flip(b[k].re, bm), flip(b[k].im, bm));
+  }
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      up[i] = ADJ ? cjmadd(u[k * 3 + i], a[k], up[i]) : cmadd(u[i * 3 + k], a[k], up[i]);
+      low[i] = ADJ ? cjmadd(u[k * 3 + i], b[k], low[i]) : cmadd(u[i * 3 + k], b[k], low[i]);
+    }
+}
 // The neighbour of a direction (0-7: mu = d / 2, forward for even d).
 __device__ __forceinline__ int neighbour_dir(const SysDesc& S, const Coord& c, int s, int d, float* eta) {
   return neighbour_rt(S, c, s, d >> 1, (d & 1) ? -1 : +1, eta);
 }
 
-// The FP64-class Wilson stencils (IEEE FP64 and double-float): two threads per
+// The FP64-class stencils (IEEE FP64 and double-float): two threads per
 // output site, one per row of the half spinor; lanes 0-15 of a warp take row 0
 // and lanes 16-31 row 1 of 16 consecutive sites, so that one load instruction
 // serves both rows' links.  Row 0 pairs with spin 3 and row 1 with spin 2 for
@@ -1232,7 +1277,9 @@ __device__ __forceinline__ int neighbour_dir(const SysDesc& S, const Coord& c, i
 //   x: c = -s i, d = s i (both rows)   y: c = d = -s (row 0), s (row 1)
 //   t: c = s, d = s (both rows)        z: c = -s i, d = s i (row 0), the opposite (row 1)
 // Blocks: T sites x RB right-hand sides, 2 T RB threads.
-template <int SPA, bool C12, bool DAG, class Epi>
+// The Laplacian runs the same way with spins row and 2 + row in a thread and no
+// projection.
+template <int SPA, bool C12, bool DAG, class Epi, int OP = OP_WILSON>
 __global__ void __launch_bounds__(512, 1)
     k_hop_rows(const __grid_constant__ Batch B, int par_mode, int link_slot, int in_slot, Epi epi, RedArgs ra) {
   static_assert(SPA == P64 || SPA == PDF, "two threads per site: FP64-class storage");
@@ -1305,16 +1352,29 @@ __global__ void __launch_bounds__(512, 1)
           }
           __syncwarp();
           const char* st = stage + (k & 1) * Ring::kStage;
-          if (k == 0) Ring::template direction<true, false>(st, row, partner, mi ^ 0x80000000u, mi, 0u, up, low);
+          if constexpr (OP == OP_LAPLACE) {
+            if (k & 1) lap_direction<C12, true>(st, row, k < 2 ? 0u : bm, up, low);
+            else lap_direction<C12, false>(st, row, k < 2 ? 0u : bm, up, low);
+          } else if (k == 0) Ring::template direction<true, false>(st, row, partner, mi ^ 0x80000000u, mi, 0u, up, low);
           else if (k == 1) Ring::template direction<true, true>(st, row, partner, mi, mi ^ 0x80000000u, 0u, up, low);
           else if (k == 2) Ring::template direction<false, false>(st, row, partner, mr, mr, bm, up, low);
           else Ring::template direction<false, true>(st, row, partner, mr ^ 0x80000000u, mr ^ 0x80000000u, bm, up, low);
           bm = next_bm;
         }
-        if (ph == 0) {
+        if (OP == OP_WILSON && ph == 0) {
 #pragma unroll
           for (int k = 0; k < 3; ++k) low[k] = other_row(low[k]);
         }
+      }
+    } else if constexpr (OP == OP_LAPLACE) {
+#pragma unroll 1
+      for (int mu = 0; mu < 4; ++mu) {
+        float ef, eb;
+        const int nf = neighbour_dir(S, c, s, 2 * mu, &ef), nb = neighbour_dir(S, c, s, 2 * mu + 1, &eb);
+        lap_direction<C12, false>(S, in, own, nf, s, row, __float_as_uint(ef) & 0x80000000u, up, low);
+        lap_direction<C12, true>(S, in, nbr, nb, nb, row, __float_as_uint(eb) & 0x80000000u, up, low);
+        own += mu_stride;
+        nbr += mu_stride;
       }
     } else {
 #pragma unroll 1

@@ -39,7 +39,8 @@ extern "C" dw_status dw_laplace_apply(const dw_field* U, const dw_field* in, dw_
   Exec E;
   E.st = st;
   std::vector<dw_lattice> lats(1, U->lat);
-  make_plan(E.P, lats, in->nrhs, 0);
+  const bool rows = in->prec == DW_F64 || in->prec == DW_DF64;  // blocks of 64 sites, as the solver's plan
+  make_plan(E.P, lats, in->nrhs, rows ? 64 : 0, rows ? 1 : 0);
   SysDesc& S = E.P.B.sd[0];
   S.f[S_LLO] = gauge_slot(U->ptr, U->lat, U->prec, U->compress12);
   S.f[S_AUX0] = spinor_slot(in);

@@ -406,8 +406,7 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
     // 808 / 733 / 723 / 723 us with 256 / 128 / 64 / 32 sites per block, IEEE FP64 is
     // the same from 128 down.
     Exec& FH = fresh.EH;
-    if (OP == OP_WILSON) make_plan(FH.P, lats, nrhs, 64, 1);
-    else FH.P = F.P;
+    make_plan(FH.P, lats, nrhs, 64, 1);
     // (k_cg_loop keeps two sets of partials; with one parity the plan has room for both)
     const int inner = (eo ? 1 : 2) * F.P.partials;
     const int partials = inner > FH.P.partials ? inner : FH.P.partials;
