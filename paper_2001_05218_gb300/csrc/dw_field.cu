@@ -499,11 +499,13 @@ static const std::string& device_name() {
   }
   return *name;
 }
-std::string tune_key(const dw_lattice* lats, int n, int nrhs, int prec, int c12) {
+// v6: shapes timed with the present kernels; v5: with those before, or written by
+// hand (the operators fall back on them).
+std::string tune_key(const dw_lattice* lats, int n, int nrhs, int prec, int c12, const char* version) {
   std::string key;
   key.reserve(64 + 24 * (size_t)n);
   key += device_name();
-  key += "/v5/";
+  key += version;
   key += prec_name(prec);
   key += c12 ? "c12/r" : "c18/r";
   key += std::to_string(nrhs);
@@ -514,6 +516,8 @@ std::string tune_key(const dw_lattice* lats, int n, int nrhs, int prec, int c12)
     }
   return key;
 }
+static std::atomic<unsigned> g_tune_gen{0};
+unsigned tune_generation() { return g_tune_gen.load(std::memory_order_acquire); }
 bool tune_lookup(const std::string& key, BlockShape* out) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
   tune_load_once();
@@ -526,6 +530,7 @@ void tune_store(const std::string& key, BlockShape v) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
   tune_load_once();
   tune_table()[key] = v;
+  g_tune_gen.fetch_add(1, std::memory_order_release);
   const std::string path = tune_path();
   const std::string dir = path.substr(0, path.find_last_of('/'));
   std::string cmd_dir = dir;

@@ -98,8 +98,9 @@ struct BlockShape {
 };
 bool tune_lookup(const std::string& key, BlockShape* out);
 void tune_store(const std::string& key, BlockShape v);
+unsigned tune_generation();  // changes with every change of the table
 // Key of the tuning cache: device name, storage, nrhs and every lattice.
-std::string tune_key(const dw_lattice* lats, int n, int nrhs, int prec, int c12);
+std::string tune_key(const dw_lattice* lats, int n, int nrhs, int prec, int c12, const char* version = "/v6/");
 
 // Stream-ordered device scratch from the library's pool (freed with
 // cudaFreeAsync), which keeps released memory between calls: from the default

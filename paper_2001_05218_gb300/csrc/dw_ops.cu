@@ -1,4 +1,6 @@
 // dw_ops.cu -- dw_apply, dw_apply_dag, dw_normal_apply.
+#include <cstring>
+
 #include "dw_apply.cuh"
 
 namespace dw {
@@ -16,10 +18,32 @@ dw_status check_op(const dw_field* U, const dw_field* in, const dw_field* out) {
 }
 
 void apply_plan(Plan& P, const dw_field* U, const dw_field* in) {
-  // untuned: the FP64-class stencils run best in blocks of 64 sites (see the solver's plan)
-  BlockShape shape{0, 0};
-  if (in->prec == DW_F64 || in->prec == DW_DF64) shape = BlockShape{64, 1};
-  tune_lookup(tune_key(&U->lat, 1, in->nrhs, U->prec, U->compress12), &shape);
+  // the thread's last lookup is kept by its values (the string keys take about 1 us)
+  struct Last {
+    unsigned generation = ~0u;
+    int dev, dims[4], nrhs, prec, c12;
+    BlockShape shape;
+  };
+  static thread_local Last last;
+  const unsigned generation = tune_generation();
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (last.generation != generation || last.dev != dev || memcmp(last.dims, U->lat.dims, sizeof last.dims) != 0 ||
+      last.nrhs != in->nrhs || last.prec != (int)U->prec || last.c12 != U->compress12) {
+    // untuned: the FP64-class stencils run best in blocks of 64 sites (see the solver's plan)
+    BlockShape shape{0, 0};
+    if (in->prec == DW_F64 || in->prec == DW_DF64) shape = BlockShape{64, 1};
+    if (!tune_lookup(tune_key(&U->lat, 1, in->nrhs, U->prec, U->compress12), &shape))
+      tune_lookup(tune_key(&U->lat, 1, in->nrhs, U->prec, U->compress12, "/v5/"), &shape);
+    last.generation = tune_generation();
+    last.dev = dev;
+    memcpy(last.dims, U->lat.dims, sizeof last.dims);
+    last.nrhs = in->nrhs;
+    last.prec = (int)U->prec;
+    last.c12 = U->compress12;
+    last.shape = shape;
+  }
+  const BlockShape shape = last.shape;
   make_plan(P, &U->lat, 1, in->nrhs, shape.T, shape.RB);
   P.pair = shape.pair;
 }
