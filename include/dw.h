@@ -144,8 +144,9 @@ dw_status dw_field_free(dw_field* f);
  * issues one copy and one kernel on `stream`.)  `host` may be pageable or
  * pinned; from pinned (page-locked) memory the copies are asynchronous and the
  * buffer must stay valid and unchanged until the stream reaches this point.
- * Staging buffers come from a memory pool owned by the library, which keeps up
- * to 8 GiB per device reserved between calls. */
+ * Staging buffers, and the temporaries of the operators, come from a memory
+ * pool owned by the library, which keeps up to 8 GiB per device reserved between
+ * calls and gives it back when an allocation of the library would fail. */
 dw_status dw_field_upload(dw_field* f, const double* host, dw_stream_t stream);
 
 /* Copy the field back to host canonical complex128 (layout kernel into a
@@ -268,8 +269,10 @@ typedef struct {
  * eo 1, compress12 0, recompute_fwd 1, tile 0, check_every 0, timeout 0,
  * verify_normal 0, outer DW_F64, defect_correction 0.
  * The CG loop runs as one CUDA graph: a device-side while-loop over the
- * iteration, with the FP64 reliable update in a conditional node; the host
- * waits once per solve.  While dw_profile_start is active the loop is stepped
+ * iteration, with the FP64 reliable update in a conditional node (on small
+ * systems the iterations between two reliable updates are one cooperative
+ * kernel, whose bounded grid barriers end the solve with DW_ERR_CUDA if they
+ * ever give up); the host waits once per solve.  While dw_profile_start is active the loop is stepped
  * from the host instead (one poll per iteration) so that every stencil launch
  * can be timed with events; the arithmetic is identical. */
 dw_status dw_solver_params_default(dw_solver_params* p);

@@ -1167,7 +1167,7 @@ __device__ __forceinline__ DF warp_sum_lane0(DF v, int from = 16) {
 // threads (T a multiple of 32); group g works on right-hand side r = y*RB + g
 // for the block's right-hand-side block y.  The producing kernel sums each
 // group's values in a fixed order (double-float on the FP32 pipes, or IEEE FP64 for FP64
-// arithmetic) and writes one IEEE-FP64 partial per block and right-hand side;
+// arithmetic) and writes one double-float partial per block and right-hand side;
 // nothing in it waits.  k_finish, launched next on the same stream (which
 // orders the partial writes before it), sums each column's partials in a
 // fixed order and runs the finalizer.  Results are bitwise reproducible.
@@ -1245,8 +1245,9 @@ struct FinPlan {
 // instead of 1024 (launching and draining 32 warps costs more than a longer
 // loop).  With rel.on the last column to finish also sets the condition of the
 // reliable-update node (a separate one-thread kernel would cost about 2 us).
-// Measured at 16^3x32 (512 partials): 4.2 us per launch before, see k_finish's
-// caller for the rule on the block size.
+// Measured at 16^3x32 (512 partials): 4.2 us per launch before, 3.3 now; 24^3x48 with
+// 12 columns of 2592 partials 5.7 and 5.5 us; see k_finish's caller for the rule on
+// the block size.
 constexpr int kFinishThreads = 1024, kFinishThreadsSmall = 256;
 // What the last column of a finishing kernel inside the graph does: on = 1 sets
 // the reliable-update node's condition; 2 and 3 count a reliable update, and 2

@@ -167,10 +167,18 @@ inline void hop(const Exec& E, int par_mode, int link_slot, In in, Epi epi, int 
   constexpr bool kRows = (SPA == P64 || SPA == PDF) && LP == SPA && std::is_same<In, InOne<SPA>>::value;
   bool launched = false;
   if constexpr (kRows) {
-    const size_t smem = SPA == PDF ? (size_t)E.P.block.x / 16 * RowRing<C12>::kBytes : 0;
-    if (smem > 48 * 1024) allow_shared(k_hop_rows<SPA, C12, DAG, Epi, OP>, smem);
-    launch(k_hop_rows<SPA, C12, DAG, Epi, OP>, E.grid(par_mode), 2 * E.P.block.x, smem, E.st, E.batch(), par_mode, link_slot,
-           in.slot, epi, E.ra(fin));
+    const unsigned n = E.P.block.x;  // T RB
+    if (E.P.pair == 2) {  // blocks of T sites, eight threads each
+      const size_t smem = (size_t)n / 4 * (SPA == PDF ? RowRing<C12>::kBytes : 3072);
+      if (smem > 48 * 1024) allow_shared(k_hop_rows<SPA, C12, DAG, Epi, OP, true>, smem);
+      launch(k_hop_rows<SPA, C12, DAG, Epi, OP, true>, E.grid(par_mode), 8 * n, smem, E.st, E.batch(), par_mode, link_slot,
+             in.slot, epi, E.ra(fin));
+    } else {
+      const size_t smem = SPA == PDF ? (size_t)n / 16 * RowRing<C12>::kBytes : 0;
+      if (smem > 48 * 1024) allow_shared(k_hop_rows<SPA, C12, DAG, Epi, OP>, smem);
+      launch(k_hop_rows<SPA, C12, DAG, Epi, OP>, E.grid(par_mode), 2 * n, smem, E.st, E.batch(), par_mode, link_slot, in.slot,
+             epi, E.ra(fin));
+    }
     launched = true;
   }
   if constexpr ((SPA == P16 || SPA == PB16) && LP == SPA && OP == OP_WILSON && std::is_same<In, InOne<SPA>>::value) {

@@ -7,7 +7,8 @@
 // kernel spin-projects the neighbour to a half spinor (2 spins x 3 colours),
 // multiplies by the link or its adjoint, and reconstructs the lower two spins
 // (the four stages of the paper's Fig. 1: load, linear combination, 3x3
-// mat-vec, accumulate).  One thread per (output site, right-hand side);
+// mat-vec, accumulate).  One thread per (output site, right-hand side) in k_hop
+// (two in FP64-class storage, k_hop_rows; four on small lattices, k_hop_split);
 // threads of a warp take consecutive even-odd site indices so every load is
 // a coalesced 16-byte (or 8-byte) access.  The boundary sign eta (-1 on links
 // crossing t = Lt-1 -> 0 when antiperiodic) is applied in the kernel, so
@@ -1279,7 +1280,11 @@ __device__ __forceinline__ int neighbour_dir(const SysDesc& S, const Coord& c, i
 // Blocks: T sites x RB right-hand sides, 2 T RB threads.
 // The Laplacian runs the same way with spins row and 2 + row in a thread and no
 // projection.
-template <int SPA, bool C12, bool DAG, class Epi, int OP = OP_WILSON>
+// SPLIT: small lattices, one warp per mu for 16 sites (blocks of T sites and one
+// right-hand side, 8 T threads); the mu sums meet in shared memory.  A launch on
+// a few hundred warps is one thread's serial chain (FP64: 432 instructions of 64
+// clocks), which this cuts to a quarter; the solver's kSplitHighSites says where.
+template <int SPA, bool C12, bool DAG, class Epi, int OP = OP_WILSON, bool SPLIT = false>
 __global__ void __launch_bounds__(512, 1)
     k_hop_rows(const __grid_constant__ Batch B, int par_mode, int link_slot, int in_slot, Epi epi, RedArgs ra) {
   static_assert(SPA == P64 || SPA == PDF, "two threads per site: FP64-class storage");
@@ -1298,11 +1303,12 @@ __global__ void __launch_bounds__(512, 1)
     par = par_mode;
   }
   const SysDesc& S = B.sd[block_system(B, b)];
-  if (RB > 1) rl = (int)threadIdx.x / (2 * T);
+  if (!SPLIT && RB > 1) rl = (int)threadIdx.x / (2 * T);
   const int r = by * RB + rl;
   const int tile = b - S.tile0;
   const int row = (threadIdx.x >> 4) & 1;
-  const int at = ((((int)threadIdx.x - rl * 2 * T) >> 5) << 4) + (threadIdx.x & 15);
+  const int mu = SPLIT ? (threadIdx.x >> 5) & 3 : 0;
+  const int at = (SPLIT ? ((int)threadIdx.x >> 7) << 4 : (((int)threadIdx.x - rl * 2 * T) >> 5) << 4) + (threadIdx.x & 15);
   const int s0 = tile * T + at;
   const bool ok = s0 < S.vh;
   // a warp works on one right-hand side: the gate is the same for all its
@@ -1321,11 +1327,71 @@ __global__ void __launch_bounds__(512, 1)
     Cx<R> up[3], low[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) up[k] = low[k] = cx((R)0, (R)0);
-    // x and y, then z and t: one copy of the code for both halves, which keeps
-    // the kernel inside the instruction cache
-    if constexpr (SPA == PDF) {
+    extern __shared__ __align__(16) char ring_[];
+    if constexpr (SPLIT) {
+      constexpr int kArea = SPA == PDF ? RowRing<C12>::kBytes : 3072;  // shared memory of a warp
+      char* area = ring_ + (threadIdx.x >> 5) * kArea;
+      float ef, eb;
+      const int nf = neighbour_dir(S, c, s, 2 * mu, &ef), nb = neighbour_dir(S, c, s, 2 * mu + 1, &eb);
+      const uint32_t bf = __float_as_uint(ef) & 0x80000000u, bb = __float_as_uint(eb) & 0x80000000u;
+      const int partner = mu < 2 ? 3 - row : 2 + row;
+      const uint32_t mi = kS ^ (mu == 0 ? 0u : row1), mr = kS ^ (mu == 1 ? row1 ^ 0x80000000u : 0u);
+      own += mu * mu_stride;
+      nbr += mu * mu_stride;
+      if constexpr (SPA == PDF) {
+        using Ring = RowRing<C12>;
+        Ring::issue(area, in, own, S.vh, nf, s);
+        Ring::issue(area + Ring::kStage, in, nbr, S.vh, nb, nb);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncwarp();
+        if constexpr (OP == OP_LAPLACE) {
+          lap_direction<C12, false>(area, row, bf, up, low);
+          lap_direction<C12, true>(area + Ring::kStage, row, bb, up, low);
+        } else if (mu == 0 || mu == 2) {
+          Ring::template direction<true, false>(area, row, partner, mi ^ 0x80000000u, mi, bf, up, low);
+          Ring::template direction<true, true>(area + Ring::kStage, row, partner, mi, mi ^ 0x80000000u, bb, up, low);
+        } else {
+          Ring::template direction<false, false>(area, row, partner, mr, mr, bf, up, low);
+          Ring::template direction<false, true>(area + Ring::kStage, row, partner, mr ^ 0x80000000u, mr ^ 0x80000000u, bb, up,
+                                                low);
+        }
+      } else if constexpr (OP == OP_LAPLACE) {
+        lap_direction<C12, false>(S, in, own, nf, s, row, bf, up, low);
+        lap_direction<C12, true>(S, in, nbr, nb, nb, row, bb, up, low);
+      } else if (mu == 0 || mu == 2) {
+        row_mu<C12, true>(S, in, own, nbr, s, nf, nb, row, partner, mi ^ 0x80000000u, mi, bf, bb, up, low, true);
+      } else {
+        row_mu<C12, false>(S, in, own, nbr, s, nf, nb, row, partner, mr, mr, bf, bb, up, low, true);
+      }
+      if (OP == OP_WILSON && mu < 2) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) low[k] = other_row(low[k]);
+      }
+      __syncwarp();  // the ring has been read
+      Cx<R>* mine = reinterpret_cast<Cx<R>*>(area) + (threadIdx.x & 31);  // [6][32], then mu + 1's and so on
+      if (mu != 0) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          mine[k * 32] = up[k];
+          mine[(3 + k) * 32] = low[k];
+        }
+      }
+      __syncthreads();
+      if (mu == 0) {
+#pragma unroll
+        for (int m = 1; m < 4; ++m) {
+          const Cx<R>* p = reinterpret_cast<const Cx<R>*>(area + m * kArea) + (threadIdx.x & 31);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            up[k] = row_add(up[k], p[k * 32]);
+            low[k] = row_add(low[k], p[(3 + k) * 32]);
+          }
+        }
+      }
+    } else if constexpr (SPA == PDF) {
+      // x and y, then z and t: one copy of the code for both halves, which keeps
+      // the kernel inside the instruction cache
       using Ring = RowRing<C12>;
-      extern __shared__ char ring_[];
       char* stage = ring_ + (threadIdx.x >> 5) * Ring::kBytes;
       float eta;
       int n = neighbour_dir(S, c, s, 0, &eta);
@@ -1407,15 +1473,20 @@ __global__ void __launch_bounds__(512, 1)
         low[k] = cx(renorm(low[k].re), renorm(low[k].im));
       }
     }
-    epi.write_rows(S, par, r, s, row, up, low, nrm, ok);
-    if (!ok) nrm = red_zero(typename RedT<R>::type());
+    if (mu == 0) {
+      epi.write_rows(S, par, r, s, row, up, low, nrm, ok);
+      if (!ok) nrm = red_zero(typename RedT<R>::type());
+    }
   }
   if constexpr (Epi::kReduce) {
     const int ntiles = par_mode == 2 ? 2 * S.tpp : S.tpp;
-    reduce_block(S, 2 * T, RB, par_mode == 2 ? par * S.tpp + tile : tile, ntiles, nrm, ra, by);
+    reduce_block(S, SPLIT ? 8 * T : 2 * T, SPLIT ? 1 : RB, par_mode == 2 ? par * S.tpp + tile : tile, ntiles, nrm, ra, by);
   }
 }
 
+// (Since k_hop runs at 64 registers it is the faster of the two on 24^3x48 with 12
+// right-hand sides, 433 against 446 us per application; this one, at 128, stays for
+// the shapes on which the tuner finds it ahead.)
 // 16-bit stencil with two right-hand sides per thread: each link is loaded,
 // and with 12-real compression its third row rebuilt, once and applied to
 // both; the two neighbour loads of a direction are in flight together.  Block:

@@ -56,7 +56,11 @@ inline long long parity_work(const std::vector<dw_lattice>& lats, int nrhs) {
 // kernel (k_cg_loop).  Beyond that its 16 warps per SM lose to the separate
 // kernels: solves with 65536 / 81920 / 131072 sites of a parity, FP16, one kernel
 // 3.16 / 4.54 / 5.25 ms, separate 3.67 / 3.84 / 4.93 ms.
-constexpr long long kSplitSites = 16384, kLoopSites = 65536;
+// The high-precision stencils run one warp per mu up to kSplitHighSites: solves
+// with FP64 / double-float corrections, without and with it, us: 128 sites of a parity
+// 1007 -> 919 / 928 -> 900, 2048 sites 1585 -> 1505 / 1512 -> 1488, 4096 sites 1710 -> 1665 /
+// 1645 -> 1647; from 8192 on equal within 1% (the FP64 pipe is full either way).
+constexpr long long kSplitSites = 16384, kLoopSites = 65536, kSplitHighSites = 4096;
 
 struct SolveArgs {
   int n;
@@ -151,8 +155,9 @@ struct CG {
   }
 
   static dw_status run(const SolveArgs& a);
+  // allow_loop = false: separate kernels also where k_cg_loop fits
   static dw_status build_graph(const Exec& E, const Exec& EH, int mode, cudaGraphExec_t* exec, int* body_kernels,
-                               int* rel_kernels);
+                               int* rel_kernels, bool allow_loop);
   static dw_status run_stepped(const Exec& E, const Exec& EH, int mode, int maxiter);
 
   // The iterations in one kernel (k_cg_loop): FP32 and 16-bit systems with blocks
@@ -215,7 +220,7 @@ dw_status CG<L, A, C12, H, OP>::launch_loop(const Exec& E, int mode, cudaGraphCo
 // loop through its own maxiter / timeout / breakdown checks.
 template <int L, int A, bool C12, int H, int OP>
 dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, const Exec& EH0, int mode, cudaGraphExec_t* exec,
-                                        int* body_kernels, int* rel_kernels) {
+                                        int* body_kernels, int* rel_kernels, bool allow_loop) {
   static thread_local CaptureStreams cs;
   const int pm = eo_mode(mode) ? 0 : 2;
   cudaGraph_t g = nullptr;
@@ -244,7 +249,9 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, const Exec& EH0, int
   const long long c0 = pr.launches;
   long long c1 = c0, c2 = c0;
   DW_CUDA(cudaStreamBeginCaptureToGraph(cs.a, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-  const bool one = loop_fits(E.P, mode);
+  int dev = 0, cooperative = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&cooperative, cudaDevAttrCooperativeLaunch, dev);
+  const bool one = allow_loop && cooperative && loop_fits(E.P, mode);
   if (one) {
     DW_TRY(launch_loop(E, mode, hr, hw));
   } else {
@@ -406,7 +413,10 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
     // 808 / 733 / 723 / 723 us with 256 / 128 / 64 / 32 sites per block, IEEE FP64 is
     // the same from 128 down.
     Exec& FH = fresh.EH;
-    make_plan(FH.P, lats, nrhs, 64, 1);
+    // On small lattices they run one warp per mu for 16 sites.
+    const bool split_high = parity_work(lats, nrhs) <= kSplitHighSites;
+    make_plan(FH.P, lats, nrhs, split_high ? 16 : 64, 1);
+    if (split_high) FH.P.pair = 2;
     // (k_cg_loop keeps two sets of partials; with one parity the plan has room for both)
     const int inner = (eo ? 1 : 2) * F.P.partials;
     const int partials = inner > FH.P.partials ? inner : FH.P.partials;
@@ -470,7 +480,13 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
     for (int i = 0; i < n; ++i) memcpy(FH.P.B.sd[i].f, F.P.B.sd[i].f, sizeof F.P.B.sd[i].f);
     FH.rb = F.rb;
     F.st = FH.st = st;
-    dw_status gs = build_graph(F, FH, mode, &fresh.exec, &fresh.body_k, &fresh.rel_k);
+    dw_status gs = build_graph(F, FH, mode, &fresh.exec, &fresh.body_k, &fresh.rel_k, true);
+    if (gs == DW_ERR_CUDA && loop_fits(F.P, mode)) {
+      // a process that may not put cooperative kernels into a conditional node
+      // (under MPS, for instance) runs the separate kernels
+      (void)cudaGetLastError();
+      gs = build_graph(F, FH, mode, &fresh.exec, &fresh.body_k, &fresh.rel_k, false);
+    }
     if (gs != DW_OK) {
       cudaFree(fresh.arena);
       return gs;
