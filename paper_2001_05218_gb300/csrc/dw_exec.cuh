@@ -85,7 +85,8 @@ struct SolveCacheEntry {
   Exec EH;  // the plan of the high-precision stencils: the same slots and buffers
   char* arena = nullptr;
   cudaGraphExec_t exec = nullptr;
-  int body_k = 0, rel_k = 0;
+  int body_k = 0, rel_k = 0;  // kernels per pass of its loop and of its reliable update
+  bool one = false;           // its iterations are k_cg_loop
   std::vector<std::pair<char*, size_t>> zero;  // ranges cleared at the start of every solve
 };
 // The entry with this key (moved to most recently used), or nullptr.

@@ -545,6 +545,13 @@ void tune_store(const std::string& key, BlockShape v) {
   }
 }
 
+static thread_local int t_refuse[kRefusals];
+bool refused(Refusal what) {
+  if (t_refuse[what] <= 0) return false;
+  --t_refuse[what];
+  return true;
+}
+
 static constexpr size_t kSolveCacheMax = 4;
 static std::list<SolveCacheEntry>& solve_cache() {
   static std::list<SolveCacheEntry> c;
@@ -580,6 +587,13 @@ using namespace dw;
 extern "C" {
 
 const char* dw_last_error(void) { return g_err; }
+
+// (declared by the tests that use it)
+dw_status dw_test_refuse(int what, int count) {
+  DW_CHECK(what >= 0 && what < kRefusals, DW_ERR_ARG, "unknown kind of failure %d", what);
+  t_refuse[what] = count;
+  return DW_OK;
+}
 
 dw_status dw_profile_start(int time_stencils) {
   Profiler& p = profiler();

@@ -110,6 +110,16 @@ dw_status scratch_alloc(char** p, size_t nb, cudaStream_t st);
 // cudaMalloc; when memory is short, what that pool keeps is given back first.
 cudaError_t device_alloc(char** p, size_t nb);
 
+// Failures that tests make on the host (dw_test_refuse, which dw.h does not
+// declare): the calling thread's next `count` attempts of a kind are reported as
+// failed instead of being made.
+enum Refusal {
+  REFUSE_LOOP_CAPTURE = 0,  // the cooperative launch, while the loop's graph is captured
+  REFUSE_LOOP_START,        // the launch of the instantiated graph
+  kRefusals
+};
+bool refused(Refusal what);
+
 // Device scratch for reductions of one plan.
 struct RedBuf {
   DF* partial = nullptr;

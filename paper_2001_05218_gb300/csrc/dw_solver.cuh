@@ -155,9 +155,9 @@ struct CG {
   }
 
   static dw_status run(const SolveArgs& a);
-  // allow_loop = false: separate kernels also where k_cg_loop fits
-  static dw_status build_graph(const Exec& E, const Exec& EH, int mode, cudaGraphExec_t* exec, int* body_kernels,
-                               int* rel_kernels, bool allow_loop);
+  // allow_loop = false: separate kernels also where k_cg_loop fits.  Fills the
+  // entry's graph, kernel counts and `one`, and leaves them as they are on an error.
+  static dw_status build_graph(SolveCacheEntry& ent, int mode, bool allow_loop);
   static dw_status run_stepped(const Exec& E, const Exec& EH, int mode, int maxiter);
 
   // The iterations in one kernel (k_cg_loop): FP32 and 16-bit systems with blocks
@@ -169,6 +169,9 @@ struct CG {
       if (P.B.sd[i].tpp * (eo_mode(mode) ? 1 : 2) > kLoopPartials) return false;
     return true;
   }
+  using LoopKernel = void (*)(Batch, RedArgs, unsigned long long, unsigned long long);
+  static LoopKernel loop_kernel(const Plan& P, int mode);
+  static int loop_grid(const Plan& P, int mode);
   static dw_status launch_loop(const Exec& E, int mode, cudaGraphConditionalHandle rel, cudaGraphConditionalHandle loop);
 };
 
@@ -180,36 +183,78 @@ struct CaptureStreams {
   }
 };
 
+// An open graph of build_graph.  Whichever way that ends, the thread's capture
+// streams are out of capture (a stream left in it would refuse every later call of
+// the thread that needs one), the graph is destroyed and the profiler is as before.
+struct GraphBuild {
+  CaptureStreams& cs;
+  Profiler& pr;
+  const bool on, timing;
+  const long long launches;
+  cudaGraph_t g = nullptr;
+  GraphBuild(CaptureStreams& c, Profiler& p) : cs(c), pr(p), on(p.on), timing(p.timing), launches(p.launches) {}
+  ~GraphBuild() {
+    for (cudaStream_t st : {cs.b, cs.a}) {
+      cudaStreamCaptureStatus state = cudaStreamCaptureStatusNone;
+      cudaGraph_t part;
+      if (cudaStreamIsCapturing(st, &state) != cudaSuccess || state != cudaStreamCaptureStatusNone)
+        cudaStreamEndCapture(st, &part);
+    }
+    if (g) cudaGraphDestroy(g);
+    (void)cudaGetLastError();  // reported by whoever returned
+    pr.on = on;
+    pr.timing = timing;
+    pr.launches = launches;
+  }
+};
+
+template <int L, int A, bool C12, int H, int OP>
+typename CG<L, A, C12, H, OP>::LoopKernel CG<L, A, C12, H, OP>::loop_kernel(const Plan& P, int mode) {
+  if constexpr (!kLoop) {
+    return nullptr;
+  } else if constexpr (OP == OP_LAPLACE) {
+    return k_cg_loop<L, A, C12, false, MODE_HERM>;
+  } else {
+    if (mode == MODE_NORMAL)
+      return P.pair == 2 ? k_cg_loop<L, A, C12, true, MODE_NORMAL> : k_cg_loop<L, A, C12, false, MODE_NORMAL>;
+    return P.pair == 2 ? k_cg_loop<L, A, C12, true, MODE_EO> : k_cg_loop<L, A, C12, false, MODE_EO>;
+  }
+}
+
+// Blocks of k_cg_loop, or 0 where they cannot all be resident (a cooperative
+// launch is refused then).  A block takes at least four 32-site items, and one
+// block runs per SM: more blocks than that only make the barriers dearer.
+template <int L, int A, bool C12, int H, int OP>
+int CG<L, A, C12, H, OP>::loop_grid(const Plan& P, int mode) {
+  int dev = 0, cooperative = 0, sms = 0, per_sm = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&cooperative, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !cooperative ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, loop_kernel(P, mode), kLoopThreads, 0) != cudaSuccess ||
+      per_sm < 1) {
+    (void)cudaGetLastError();
+    return 0;
+  }
+  const int items = P.B.ntot * P.nrhs * (eo_mode(mode) ? 1 : 2);
+  return (items + 3) / 4 < sms ? (items + 3) / 4 : sms;
+}
+
 template <int L, int A, bool C12, int H, int OP>
 dw_status CG<L, A, C12, H, OP>::launch_loop(const Exec& E, int mode, cudaGraphConditionalHandle rel,
                                             cudaGraphConditionalHandle loop) {
-  if constexpr (kLoop) {
-    // a block takes at least four 32-site items, and one block runs per SM: more
-    // blocks than that only make the barriers dearer
-    int dev = 0, sms = 0;
-    DW_CUDA(cudaGetDevice(&dev));
-    DW_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int items = E.P.B.ntot * E.P.nrhs * (eo_mode(mode) ? 1 : 2);
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeCooperative;
-    at[0].val.cooperative = 1;
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)((items + 3) / 4 < sms ? (items + 3) / 4 : sms));
-    lc.blockDim = dim3(kLoopThreads);
-    lc.stream = E.st;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    count_launch();
-    void (*k)(Batch, RedArgs, unsigned long long, unsigned long long) = nullptr;
-    if constexpr (OP == OP_LAPLACE) {
-      k = k_cg_loop<L, A, C12, false, MODE_HERM>;
-    } else if (mode == MODE_NORMAL) {
-      k = E.P.pair == 2 ? k_cg_loop<L, A, C12, true, MODE_NORMAL> : k_cg_loop<L, A, C12, false, MODE_NORMAL>;
-    } else {
-      k = E.P.pair == 2 ? k_cg_loop<L, A, C12, true, MODE_EO> : k_cg_loop<L, A, C12, false, MODE_EO>;
-    }
-    DW_CUDA(cudaLaunchKernelEx(&lc, k, E.P.B, E.ra(FIN_STORE0), (unsigned long long)rel, (unsigned long long)loop));
-  }
+  if (refused(REFUSE_LOOP_CAPTURE)) return set_error(DW_ERR_CUDA, "cooperative launch refused");
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3((unsigned)loop_grid(E.P, mode));
+  lc.blockDim = dim3(kLoopThreads);
+  lc.stream = E.st;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  count_launch();
+  DW_CUDA(cudaLaunchKernelEx(&lc, loop_kernel(E.P, mode), E.P.B, E.ra(FIN_STORE0), (unsigned long long)rel,
+                             (unsigned long long)loop));
   return DW_OK;
 }
 
@@ -219,12 +264,11 @@ dw_status CG<L, A, C12, H, OP>::launch_loop(const Exec& E, int mode, cudaGraphCo
 // the loop is capped at maxiter + 2 passes, and every column also leaves the
 // loop through its own maxiter / timeout / breakdown checks.
 template <int L, int A, bool C12, int H, int OP>
-dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, const Exec& EH0, int mode, cudaGraphExec_t* exec,
-                                        int* body_kernels, int* rel_kernels, bool allow_loop) {
+dw_status CG<L, A, C12, H, OP>::build_graph(SolveCacheEntry& ent, int mode, bool allow_loop) {
   static thread_local CaptureStreams cs;
   const int pm = eo_mode(mode) ? 0 : 2;
-  cudaGraph_t g = nullptr;
-  cudaGraphExec_t ge = nullptr;
+  GraphBuild build(cs, profiler());
+  cudaGraph_t& g = build.g;
   DW_CUDA(cudaGraphCreate(&g, 0));
   cudaGraphConditionalHandle hw, hr;
   DW_CUDA(cudaGraphConditionalHandleCreate(&hw, g, 1, cudaGraphCondAssignDefault));
@@ -238,20 +282,17 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, const Exec& EH0, int
   cudaGraph_t body = wp.conditional.phGraph_out[0];
   DW_CUDA(cudaGraphConditionalHandleCreate(&hr, body, 0, cudaGraphCondAssignDefault));
 
-  Exec E = E0;
+  Exec E = ent.E;
   E.st = cs.a;
   // count the captured kernel nodes (and never record profiling events into
   // the graph: events cannot live inside conditional nodes)
   Profiler& pr = profiler();
-  const bool was_on = pr.on, was_timing = pr.timing;
   pr.on = true;
   pr.timing = false;
   const long long c0 = pr.launches;
   long long c1 = c0, c2 = c0;
+  const bool one = allow_loop && loop_fits(E.P, mode) && loop_grid(E.P, mode) > 0;
   DW_CUDA(cudaStreamBeginCaptureToGraph(cs.a, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-  int dev = 0, cooperative = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&cooperative, cudaDevAttrCooperativeLaunch, dev);
-  const bool one = allow_loop && cooperative && loop_fits(E.P, mode);
   if (one) {
     DW_TRY(launch_loop(E, mode, hr, hw));
   } else {
@@ -293,7 +334,7 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, const Exec& EH0, int
     c1 = pr.launches;
     DW_CUDA(cudaStreamBeginCaptureToGraph(cs.b, ip.conditional.phGraph_out[0], nullptr, nullptr, 0,
                                           cudaStreamCaptureModeThreadLocal));
-    Exec RH = EH0;
+    Exec RH = ent.EH;
     RH.st = cs.b;
     reliable(R, RH, mode, one ? RelCond{(unsigned long long)hw, 2} : RelCond{0, 3});
     cudaGraph_t tmp;
@@ -308,22 +349,15 @@ dw_status CG<L, A, C12, H, OP>::build_graph(const Exec& E0, const Exec& EH0, int
   }
   cudaGraph_t tmp;
   DW_CUDA(cudaStreamEndCapture(cs.a, &tmp));
-  cudaError_t e = cudaGraphInstantiate(&ge, g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) {
-    pr.on = was_on;
-    pr.timing = was_timing;
-    pr.launches = c0;
-    return cuda_error(e, "CG graph", __FILE__, __LINE__);
-  }
-  *exec = ge;
+  cudaGraphExec_t ge = nullptr;
+  DW_CUDA(cudaGraphInstantiate(&ge, g, 0));
+  if (ent.exec) cudaGraphExecDestroy(ent.exec);
+  ent.exec = ge;
+  ent.one = one;
   // kernel nodes per pass of the loop body and of the reliable-update branch;
   // the executed counts are added once the device counters are read back
-  *body_kernels = (int)((c1 - c0) + (pr.launches - c2));
-  *rel_kernels = (int)(c2 - c1);
-  pr.launches = c0;
-  pr.on = was_on;
-  pr.timing = was_timing;
+  ent.body_k = (int)((c1 - c0) + (pr.launches - c2));
+  ent.rel_k = (int)(c2 - c1);
   return DW_OK;
 }
 
@@ -480,13 +514,10 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
     for (int i = 0; i < n; ++i) memcpy(FH.P.B.sd[i].f, F.P.B.sd[i].f, sizeof F.P.B.sd[i].f);
     FH.rb = F.rb;
     F.st = FH.st = st;
-    dw_status gs = build_graph(F, FH, mode, &fresh.exec, &fresh.body_k, &fresh.rel_k, true);
-    if (gs == DW_ERR_CUDA && loop_fits(F.P, mode)) {
-      // a process that may not put cooperative kernels into a conditional node
-      // (under MPS, for instance) runs the separate kernels
-      (void)cudaGetLastError();
-      gs = build_graph(F, FH, mode, &fresh.exec, &fresh.body_k, &fresh.rel_k, false);
-    }
+    // a process that may not put cooperative kernels into a conditional node
+    // (under MPS, for instance) runs the separate kernels
+    dw_status gs = build_graph(fresh, mode, true);
+    if (gs == DW_ERR_CUDA && loop_fits(F.P, mode)) gs = build_graph(fresh, mode, false);
     if (gs != DW_OK) {
       cudaFree(fresh.arena);
       return gs;
@@ -567,10 +598,16 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
   DW_CUDA(cudaGetLastError());
 
   // ---- iterations
-  const int body_k = ent->body_k, rel_k = ent->rel_k;
   const bool graph = !profiler().timing;
   if (graph) {
-    DW_CUDA(cudaGraphLaunch(ent->exec, st));
+    cudaError_t e = ent->one && refused(REFUSE_LOOP_START) ? cudaErrorCooperativeLaunchTooLarge
+                                                           : cudaGraphLaunch(ent->exec, st);
+    if (e != cudaSuccess && ent->one) {  // as above, refused only now: this plan goes on with the separate kernels
+      (void)cudaGetLastError();
+      DW_TRY(build_graph(*ent, mode, false));
+      e = cudaGraphLaunch(ent->exec, st);
+    }
+    DW_CUDA(e);
   } else {
     DW_TRY(run_stepped(E, EH, mode, a.p.maxiter));
   }
@@ -617,7 +654,7 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
   DW_CUDA(cudaMemcpyAsync(hc.data(), E.rb.cols, sizeof(ColState) * hc.size(), cudaMemcpyDeviceToHost, st));
   DW_CUDA(cudaMemcpyAsync(&hf, E.rb.flags, sizeof hf, cudaMemcpyDeviceToHost, st));
   DW_CUDA(cudaStreamSynchronize(st));
-  if (graph && profiler().on) profiler().launches += (long long)hf.loops * body_k + (long long)hf.rel_runs * rel_k;
+  if (graph && profiler().on) profiler().launches += (long long)hf.loops * ent->body_k + (long long)hf.rel_runs * ent->rel_k;
   float ms = 0.f;
   cudaEventElapsedTime(&ms, ev0, ev1);
   cudaEventDestroy(ev0);

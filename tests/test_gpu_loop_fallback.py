@@ -1,0 +1,60 @@
+"""Small solves where the one-kernel CG loop cannot run: the same solve with the
+separate kernels, and nothing left behind for the thread's next solves.  The
+failures are made on the host (dw_test_refuse)."""
+import ctypes
+
+import numpy as np
+import pytest
+
+from paper_2001_05218_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+LOOP_CAPTURE, LOOP_START = 0, 1  # kinds of failure, as in csrc/dw_internal.h
+DIMS, KAPPA = (8, 8, 8, 16), 0.12
+
+
+@pytest.fixture(scope="module")
+def dw():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_2001_05218_gb300 import dw as m
+    return m
+
+
+def _refuse(dw, what, count):
+    assert ctypes.CDLL(dw.LIB_PATH).dw_test_refuse(what, count) == dw.DW_OK
+
+
+def _solve(dw, keep, U, b, **kw):
+    """A solve on fields of its own (kept, so that no plan of another solve fits):
+    status, solution, iterations, kernels launched."""
+    Ug, bg, xg = dw.gauge(DIMS, KAPPA, U), dw.spinor(DIMS, b), dw.spinor(DIMS)
+    keep.append((Ug, bg, xg))
+    dw.profile_start(time_stencils=False)
+    try:
+        s, st = dw.cg_solve(Ug, bg, xg, dw.params(tol=1e-10, **kw))
+    finally:
+        _, launches = dw.profile_stop()
+    assert s == dw.DW_OK and st[0]["true_rel_resid"] <= 1e-10
+    return xg.download(), st[0]["iters"], launches
+
+
+@pytest.mark.parametrize("what", [LOOP_CAPTURE, LOOP_START])
+@pytest.mark.parametrize("kw", [dict(inner="f16", compress12=1, outer="df64"), dict(inner="f32")])
+def test_refused_cooperative_launch_falls_back(dw, what, kw):
+    U, b = I.gauge_field(DIMS, "exp", 71, 1, 0.4), I.gaussian_spinor(DIMS, 71, 2)
+    keep = []
+    x0, n0, l0 = _solve(dw, keep, U, b, **kw)
+    _refuse(dw, what, 1)
+    try:
+        x1, n1, l1 = _solve(dw, keep, U, b, **kw)
+    finally:
+        _refuse(dw, what, 0)
+    # the separate kernels give the one kernel's results bit by bit; nine or more
+    # launches per iteration show that they ran
+    assert n1 == n0 and np.array_equal(x1, x0)
+    assert l0 < 4 * n0 < l1
+    # the thread's next plan: captured anew, in one kernel again
+    x2, n2, l2 = _solve(dw, keep, U, b, **kw)
+    assert n2 == n0 and np.array_equal(x2, x0) and l2 == l0
