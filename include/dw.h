@@ -269,10 +269,15 @@ typedef struct {
  * eo 1, compress12 0, recompute_fwd 1, tile 0, check_every 0, timeout 0,
  * verify_normal 0, outer DW_F64, defect_correction 0.
  * The CG loop runs as one CUDA graph: a device-side while-loop over the
- * iteration, with the FP64 reliable update in a conditional node (on small
- * systems the iterations between two reliable updates are one cooperative
- * kernel, whose bounded grid barriers end the solve with DW_ERR_CUDA if they
- * ever give up); the host waits once per solve.  While dw_profile_start is active the loop is stepped
+ * iteration, with the FP64 reliable update in a conditional node; the host
+ * waits once per solve.  On small systems the iterations between two reliable
+ * updates are one cooperative kernel: it starts when all its blocks (one per
+ * SM, each with all of its registers) fit on the GPU at once, so beside other
+ * work on the GPU such a solve waits for SMs to come free, and its grid barriers
+ * are bounded.  Where the launch is refused the solve runs the
+ * separate kernels instead; if a barrier ever gives up, it goes on with them
+ * from the x that the last reliable update left (iters, time_ms and maxiter then
+ * count from there).  While dw_profile_start is active the loop is stepped
  * from the host instead (one poll per iteration) so that every stencil launch
  * can be timed with events; the arithmetic is identical. */
 dw_status dw_solver_params_default(dw_solver_params* p);

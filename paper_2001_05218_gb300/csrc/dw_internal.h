@@ -116,6 +116,7 @@ cudaError_t device_alloc(char** p, size_t nb);
 enum Refusal {
   REFUSE_LOOP_CAPTURE = 0,  // the cooperative launch, while the loop's graph is captured
   REFUSE_LOOP_START,        // the launch of the instantiated graph
+  REFUSE_LOOP_WAIT,         // every wait of a loop kernel's grid barriers beyond the first look
   kRefusals
 };
 bool refused(Refusal what);

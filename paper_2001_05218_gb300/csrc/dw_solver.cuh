@@ -169,7 +169,7 @@ struct CG {
       if (P.B.sd[i].tpp * (eo_mode(mode) ? 1 : 2) > kLoopPartials) return false;
     return true;
   }
-  using LoopKernel = void (*)(Batch, RedArgs, unsigned long long, unsigned long long);
+  using LoopKernel = void (*)(Batch, RedArgs, unsigned long long, unsigned long long, int);
   static LoopKernel loop_kernel(const Plan& P, int mode);
   static int loop_grid(const Plan& P, int mode);
   static dw_status launch_loop(const Exec& E, int mode, cudaGraphConditionalHandle rel, cudaGraphConditionalHandle loop);
@@ -254,7 +254,7 @@ dw_status CG<L, A, C12, H, OP>::launch_loop(const Exec& E, int mode, cudaGraphCo
   lc.numAttrs = 1;
   count_launch();
   DW_CUDA(cudaLaunchKernelEx(&lc, loop_kernel(E.P, mode), E.P.B, E.ra(FIN_STORE0), (unsigned long long)rel,
-                             (unsigned long long)loop));
+                             (unsigned long long)loop, refused(REFUSE_LOOP_WAIT) ? 0 : kBarrierPolls));
   return DW_OK;
 }
 
@@ -392,6 +392,7 @@ dw_status CG<L, A, C12, H, OP>::run_stepped(const Exec& E, const Exec& EH, int m
 
 template <int L, int A, bool C12, int H, int OP>
 dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
+  const auto t0 = std::chrono::steady_clock::now();
   const int n = a.n;
   const int mode = a.mode;
   const int nrhs = a.b[0]->nrhs;
@@ -660,7 +661,19 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
   cudaEventDestroy(ev0);
   cudaEventDestroy(ev1);
   DW_CUDA(cudaGetLastError());
-  if (hf.bar_error) return set_error(DW_ERR_CUDA, "a grid barrier of the CG loop gave up waiting");
+  if (hf.bar_error) {
+    // A grid barrier gave up: x is as the last reliable update left it (increments
+    // enter it there only), so the solve goes on from it, with the separate kernels
+    // and what is left of the time budget.
+    DW_CHECK(ent->one, DW_ERR_CUDA, "a grid barrier of the CG loop gave up waiting");
+    DW_TRY(build_graph(*ent, mode, false));
+    SolveArgs again = a;
+    if (a.p.timeout_s > 0) {
+      const std::chrono::duration<double> spent = std::chrono::steady_clock::now() - t0;
+      again.p.timeout_s = a.p.timeout_s > spent.count() + 1e-6 ? a.p.timeout_s - spent.count() : 1e-6;
+    }
+    return run(again);
+  }
 
   // ---- statistics
   dw_status worst = DW_OK;

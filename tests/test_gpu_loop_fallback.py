@@ -6,11 +6,12 @@ import ctypes
 import numpy as np
 import pytest
 
+from oracle import oracle as O
 from paper_2001_05218_gb300 import inputs as I
 
 pytestmark = pytest.mark.gpu
 
-LOOP_CAPTURE, LOOP_START = 0, 1  # kinds of failure, as in csrc/dw_internal.h
+LOOP_CAPTURE, LOOP_START, LOOP_WAIT = 0, 1, 2  # kinds of failure, as in csrc/dw_internal.h
 DIMS, KAPPA = (8, 8, 8, 16), 0.12
 
 
@@ -56,5 +57,30 @@ def test_refused_cooperative_launch_falls_back(dw, what, kw):
     assert n1 == n0 and np.array_equal(x1, x0)
     assert l0 < 4 * n0 < l1
     # the thread's next plan: captured anew, in one kernel again
+    x2, n2, l2 = _solve(dw, keep, U, b, **kw)
+    assert n2 == n0 and np.array_equal(x2, x0) and l2 == l0
+
+
+@pytest.mark.parametrize("kw", [dict(inner="f16", compress12=1, outer="df64"), dict(inner="f32"),
+                                dict(inner="f32", timeout_s=60.0)])
+def test_barrier_that_gives_up_is_followed_by_the_separate_kernels(dw, kw):
+    """32 blocks whose barriers give up after one look: all but the last block to
+    arrive leave (the waits are bounded by the same count)."""
+    U, b = I.gauge_field(DIMS, "exp", 72, 1, 0.4), I.gaussian_spinor(DIMS, 72, 2)
+    keep = []
+    x0, n0, l0 = _solve(dw, keep, U, b, **kw)
+    _refuse(dw, LOOP_WAIT, 1)
+    try:
+        x1, n1, l1 = _solve(dw, keep, U, b, **kw)
+    finally:
+        _refuse(dw, LOOP_WAIT, 0)
+    r = O.dirac(DIMS, KAPPA, U, x1) - b
+    assert np.linalg.norm(r) <= 1e-10 * np.linalg.norm(b)
+    assert l0 < 4 * n0 < l1
+    # the plan goes on without the one kernel
+    Ug, bg, xg = keep[1]
+    xg.storage.zero_()
+    s, st = dw.cg_solve(Ug, bg, xg, dw.params(tol=1e-10, **kw))
+    assert s == dw.DW_OK and st[0]["iters"] == n0 and np.array_equal(xg.download(), x0)
     x2, n2, l2 = _solve(dw, keep, U, b, **kw)
     assert n2 == n0 and np.array_equal(x2, x0) and l2 == l0
