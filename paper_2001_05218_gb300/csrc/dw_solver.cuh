@@ -56,11 +56,20 @@ inline long long parity_work(const std::vector<dw_lattice>& lats, int nrhs) {
 // kernel (k_cg_loop).  Beyond that its 16 warps per SM lose to the separate
 // kernels: solves with 65536 / 81920 / 131072 sites of a parity, FP16, one kernel
 // 3.16 / 4.54 / 5.25 ms, separate 3.67 / 3.84 / 4.93 ms.
+// Where blocks of 32 sites and one right-hand side are given (tile, the tuner), the
+// one kernel goes up to kLoopSites too, and up to kLoopSitesFew with at most
+// kFewCols columns, whose partials every block sums.  Solves, one kernel /
+// separate kernels in those blocks, ms: 98304 sites in 12 columns, FP32 4.76 / 4.08,
+// FP16 4.85 / 3.98; 196608 in 6, FP32 6.81 / 6.58; 262144 in 4, FP16 9.33 / 7.78;
+// 131072 in 2, FP32 4.81 / 5.40, FP16 4.40 / 4.57, normal equations FP32 6.66 / 7.75,
+// Laplacian FP32 2.46 / 2.66; 131072 in 4, FP32 4.53 / 4.79, FP16 4.40 / 4.38.
 // The high-precision stencils run one warp per mu up to kSplitHighSites: solves
 // with FP64 / double-float corrections, without and with it, us: 128 sites of a parity
 // 1007 -> 919 / 928 -> 900, 2048 sites 1585 -> 1505 / 1512 -> 1488, 4096 sites 1710 -> 1665 /
 // 1645 -> 1647; from 8192 on equal within 1% (the FP64 pipe is full either way).
 constexpr long long kSplitSites = 16384, kLoopSites = 65536, kSplitHighSites = 4096;
+constexpr long long kLoopSitesFew = 131072;
+constexpr int kFewCols = 4;
 
 struct SolveArgs {
   int n;
@@ -160,14 +169,17 @@ struct CG {
   static dw_status build_graph(SolveCacheEntry& ent, int mode, bool allow_loop);
   static dw_status run_stepped(const Exec& E, const Exec& EH, int mode, int maxiter);
 
-  // The iterations in one kernel (k_cg_loop): FP32 and 16-bit systems with blocks
-  // of 32 sites, few enough columns and tiles for its sums.
+  // The iterations in one kernel (k_cg_loop): FP32 and 16-bit systems of the sizes
+  // above with blocks of 32 sites and few enough columns and tiles for its sums.
   static constexpr bool kLoop = L != P64 && L != PDF;
   static bool loop_fits(const Plan& P, int mode) {
     if (!kLoop || mode == MODE_FULL || P.B.T != 32 || P.B.RB != 1 || P.ncols > kLoopCols) return false;
-    for (int i = 0; i < P.nsys; ++i)
+    long long work = 0;  // the size decides whoever chose the blocks: this rule, the tuner or the caller (tile)
+    for (int i = 0; i < P.nsys; ++i) {
       if (P.B.sd[i].tpp * (eo_mode(mode) ? 1 : 2) > kLoopPartials) return false;
-    return true;
+      work += (long long)P.B.sd[i].vh * P.nrhs * (eo_mode(mode) ? 1 : 2);
+    }
+    return work <= (P.ncols <= kFewCols ? kLoopSitesFew : kLoopSites);
   }
   using LoopKernel = void (*)(Batch, RedArgs, unsigned long long, unsigned long long, int);
   static LoopKernel loop_kernel(const Plan& P, int mode);

@@ -84,3 +84,39 @@ def test_barrier_that_gives_up_is_followed_by_the_separate_kernels(dw, kw):
     assert s == dw.DW_OK and st[0]["iters"] == n0 and np.array_equal(xg.download(), x0)
     x2, n2, l2 = _solve(dw, keep, U, b, **kw)
     assert n2 == n0 and np.array_equal(x2, x0) and l2 == l0
+
+
+@pytest.mark.parametrize("op,dims,n,nrhs,one", [
+    ("wilson", (8, 8, 16, 16), 1, 8, True),      # 65536 sites x right-hand sides in all
+    ("wilson", (8, 8, 16, 16), 1, 12, False),    # 98304
+    ("wilson", (16, 16, 16, 16), 4, 1, True),    # four lattices, 131072
+    ("wilson", (16, 16, 16, 16), 5, 1, False),
+    ("normal", (16, 16, 16, 16), 1, 2, True),    # 131072 with both parities
+    ("normal", (16, 16, 16, 16), 1, 3, False),
+    ("laplace", (8, 8, 16, 16), 1, 12, False),
+])
+def test_one_kernel_rule_counts_all_sites(dw, op, dims, n, nrhs, one):
+    """With 32-site blocks, which a caller may ask for (tile) and the tuner may
+    find fastest, the line lies at 65536 sites x right-hand sides x parities, and
+    at 131072 with at most four columns."""
+    Us, bs, xs = [], [], []
+    for i in range(n):
+        U = I.gauge_field(dims, "exp", 73 + i, 1, 0.4)
+        b = np.stack([I.gaussian_spinor(dims, 73 + i, 2 + r) for r in range(nrhs)])
+        Us.append(dw.gauge(dims, 0.11, U))
+        bs.append(dw.spinor(dims, b if nrhs > 1 else b[0], nrhs=nrhs))
+        xs.append(dw.spinor(dims, nrhs=nrhs))
+    p = dw.params(tol=1e-10, inner="f32", outer="df64", tile=32)
+    dw.profile_start(time_stencils=False)
+    try:
+        if n > 1:
+            s, st = dw.cg_solve_batched(Us, bs, xs, p)
+        else:
+            solve = {"wilson": dw.cg_solve, "normal": dw.cg_solve_normal, "laplace": dw.cg_solve_laplace}[op]
+            s, st = solve(Us[0], bs[0], xs[0], p)
+    finally:
+        _, launches = dw.profile_stop()
+    iters = max(v["iters"] for v in st)
+    assert s == dw.DW_OK and max(v["true_rel_resid"] for v in st) <= 1e-10
+    # the separate kernels are six or more launches per iteration
+    assert (launches < 3 * iters + 20) == one, (launches, iters)
