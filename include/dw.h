@@ -146,7 +146,8 @@ dw_status dw_field_free(dw_field* f);
  * buffer must stay valid and unchanged until the stream reaches this point.
  * Staging buffers, and the temporaries of the operators, come from a memory
  * pool owned by the library, which keeps up to 8 GiB per device reserved between
- * calls and gives it back when an allocation of the library would fail. */
+ * calls and gives it back when an allocation of the library would fail (other
+ * allocators of the process cannot have it until then). */
 dw_status dw_field_upload(dw_field* f, const double* host, dw_stream_t stream);
 
 /* Copy the field back to host canonical complex128 (layout kernel into a

@@ -770,6 +770,13 @@ static dw_status staging_pool(cudaMemPool_t* out) {
   return DW_OK;
 }
 
+// After an allocation failed: waits for the frees that are under way and hands what
+// the pool keeps back to the driver.
+static bool pool_gives_back(cudaMemPool_t pool) {
+  (void)cudaGetLastError();
+  return cudaDeviceSynchronize() == cudaSuccess && cudaMemPoolTrimTo(pool, 0) == cudaSuccess;
+}
+
 }  // extern "C"
 dw_status dw::scratch_alloc(char** p, size_t nb, cudaStream_t st) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -779,18 +786,18 @@ dw_status dw::scratch_alloc(char** p, size_t nb, cudaStream_t st) {
   }
   cudaMemPool_t pool;
   DW_TRY(staging_pool(&pool));
-  DW_CUDA(cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), nb, pool, st));
+  cudaError_t e = refused(REFUSE_SCRATCH) ? cudaErrorMemoryAllocation
+                                          : cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), nb, pool, st);
+  if (e == cudaErrorMemoryAllocation && pool_gives_back(pool))
+    e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), nb, pool, st);
+  DW_CUDA(e);
   return DW_OK;
 }
 cudaError_t dw::device_alloc(char** p, size_t nb) {
   cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), nb);
-  if (e == cudaErrorMemoryAllocation) {
-    cudaMemPool_t pool;
-    (void)cudaGetLastError();
-    if (staging_pool(&pool) == DW_OK && cudaDeviceSynchronize() == cudaSuccess &&
-        cudaMemPoolTrimTo(pool, 0) == cudaSuccess)
-      e = cudaMalloc(reinterpret_cast<void**>(p), nb);
-  }
+  cudaMemPool_t pool;
+  if (e == cudaErrorMemoryAllocation && staging_pool(&pool) == DW_OK && pool_gives_back(pool))
+    e = cudaMalloc(reinterpret_cast<void**>(p), nb);
   return e;
 }
 extern "C" {

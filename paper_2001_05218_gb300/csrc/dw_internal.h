@@ -117,6 +117,7 @@ enum Refusal {
   REFUSE_LOOP_CAPTURE = 0,  // the cooperative launch, while the loop's graph is captured
   REFUSE_LOOP_START,        // the launch of the instantiated graph
   REFUSE_LOOP_WAIT,         // every wait of a loop kernel's grid barriers beyond the first look
+  REFUSE_SCRATCH,           // the first attempt of an allocation from the library's pool
   kRefusals
 };
 bool refused(Refusal what);

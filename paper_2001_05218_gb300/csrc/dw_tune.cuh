@@ -60,7 +60,7 @@ BlockShape tune_inner_shape(const std::vector<dw_lattice>& lats, int nrhs, const
   }
   const size_t red_b = part_b + cols_b + al(sizeof(Flags));
   char* buf = nullptr;
-  if (cudaMallocAsync((void**)&buf, 3 * per + red_b, st) != cudaSuccess) return BlockShape{0, 0};
+  if (scratch_alloc(&buf, 3 * per + red_b, st) != DW_OK) return BlockShape{0, 0};
   cudaMemsetAsync(buf, 0, 3 * per + red_b, st);
   RedBuf rb;
   rb.partial = reinterpret_cast<DF*>(buf + 3 * per);
