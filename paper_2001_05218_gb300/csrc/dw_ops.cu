@@ -35,7 +35,7 @@ void apply_plan(Plan& P, const dw_field* U, const dw_field* in) {
     if (in->prec == DW_F64 || in->prec == DW_DF64) shape = BlockShape{64, 1};
     if (!tune_lookup(tune_key(&U->lat, 1, in->nrhs, U->prec, U->compress12), &shape))
       tune_lookup(tune_key(&U->lat, 1, in->nrhs, U->prec, U->compress12, "/v5/"), &shape);
-    last.generation = tune_generation();
+    last.generation = generation;  // as before the lookup: a record stored since then is looked up next time
     last.dev = dev;
     memcpy(last.dims, U->lat.dims, sizeof last.dims);
     last.nrhs = in->nrhs;
