@@ -145,31 +145,6 @@ __device__ __forceinline__ DF add_lazy(DF a, DF b) {
 }
 __device__ __forceinline__ DF renorm(DF a) { return fast_two_sum(a.hi, a.lo); }
 
-// Exact high product and its low-order terms: x*y = p + e (+ x.lo*y.lo).
-__device__ __forceinline__ DF prod_terms(DF x, DF y) {
-  const float p = __fmul_rn(x.hi, y.hi);
-  float e = __fmaf_rn(x.hi, y.hi, -p);
-  e = __fmaf_rn(x.hi, y.lo, e);
-  e = __fmaf_rn(x.lo, y.hi, e);
-  return df_make(p, e);
-}
-
-// Sum of 6 products x_i * y_i: exact high products added pairwise with TwoSum
-// (a tree, so the three first-level sums are independent), all low-order
-// terms collected in FP32, one renormalisation.
-__device__ __forceinline__ DF df_dot6(const DF (&x)[6], const DF (&y)[6]) {
-  const DF a = prod_terms(x[0], y[0]), b = prod_terms(x[1], y[1]), c = prod_terms(x[2], y[2]);
-  const DF d = prod_terms(x[3], y[3]), e = prod_terms(x[4], y[4]), f = prod_terms(x[5], y[5]);
-  const DF ab = two_sum(a.hi, b.hi), cd = two_sum(c.hi, d.hi), ef = two_sum(e.hi, f.hi);
-  const DF abcd = two_sum(ab.hi, cd.hi);
-  const DF all = two_sum(abcd.hi, ef.hi);
-  const float lo1 = __fadd_rn(__fadd_rn(a.lo, b.lo), __fadd_rn(c.lo, d.lo));
-  const float lo2 = __fadd_rn(__fadd_rn(e.lo, f.lo), __fadd_rn(ab.lo, cd.lo));
-  const float lo3 = __fadd_rn(__fadd_rn(ef.lo, abcd.lo), all.lo);
-  return fast_two_sum(all.hi, __fadd_rn(__fadd_rn(lo1, lo2), lo3));
-}
-
-
 // Two independent double-float numbers in the two lanes of packed FP32x2
 // registers: each instruction below does the same IEEE operation on both
 // lanes (Blackwell's fma/add/mul.rn.f32x2), so one sequence computes two
@@ -194,7 +169,9 @@ __device__ __forceinline__ void prod_terms2(DF x, const DF2& y, float2& p, float
   e = __ffma2_rn(xh, y.lo, e);
   e = __ffma2_rn(bc2(x.lo), y.hi, e);
 }
-// Two six-term dot products sum_i x_i * y_i (lane-wise in y), as df_dot6.
+// Two six-term dot products sum_i x_i * y_i (lane-wise in y): exact high products
+// x.hi*y.hi added with TwoSum (a tree, so the three first-level sums are
+// independent), all low-order terms collected in FP32, one renormalisation.
 __device__ __forceinline__ DF2 df2_dot6(const DF (&x)[6], const DF2 (&y)[6]) {
   float2 p[6], e[6];
 #pragma unroll
@@ -920,7 +897,8 @@ constexpr int kMaxSys = 8;
 struct Batch {
   int nsys;  // systems in this launch
   int ntot;  // blocks per parity over all systems (grid x per parity)
-  int T;     // sites per block (per right-hand side), multiple of 32
+  int T;     // sites per block (per right-hand side), multiple of 32; 16 only where
+             // every launch is k_hop_rows in its one-warp-per-mu form
   int RB;    // right-hand sides per block
   int ny;    // right-hand-side blocks, ceil(nrhs / RB): the grid is x = (parity
              // range, tile, rhs block) with the rhs block varying fastest

@@ -212,10 +212,6 @@ __device__ __forceinline__ void su3_mul_w(const uint32_t (&u)[9], const uint32_t
 // Double-float version: each real output is one 6-term dot product.  The two
 // spin rows of the half spinor are the two lanes of packed FP32x2 arithmetic,
 // so each packed dot product yields one real output for both rows.
-#ifndef DW_DF_PACKED
-#define DW_DF_PACKED 1
-#endif
-#if DW_DF_PACKED
 template <bool ADJ>
 __device__ __forceinline__ void su3_mul(const Cx<DF> (&u)[9], const Cx<DF> (&h)[6], Cx<DF> (&g)[6]) {
   DF2 hr[3], hi[3], hrn[3], hin[3];  // rows k = 0, 1 in the lanes; n: negated
@@ -254,33 +250,6 @@ __device__ __forceinline__ void su3_mul(const Cx<DF> (&u)[9], const Cx<DF> (&h)[
     g[3 + a].im = df_make(im.hi.y, im.lo.y);
   }
 }
-#else
-template <bool ADJ>
-__device__ __forceinline__ void su3_mul(const Cx<DF> (&u)[9], const Cx<DF> (&h)[6], Cx<DF> (&g)[6]) {
-#pragma unroll
-  for (int k = 0; k < 2; ++k)
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      DF xr[6], yr[6], xi[6], yi[6];
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const Cx<DF> m = ADJ ? u[b * 3 + a] : u[a * 3 + b];
-        const Cx<DF> v = h[3 * k + b];
-        // re = m.re v.re -/+ m.im v.im ; im = m.re v.im +/- m.im v.re  (lower sign: adjoint)
-        xr[2 * b] = m.re;
-        yr[2 * b] = v.re;
-        xr[2 * b + 1] = ADJ ? m.im : -m.im;
-        yr[2 * b + 1] = v.im;
-        xi[2 * b] = m.re;
-        yi[2 * b] = v.im;
-        xi[2 * b + 1] = ADJ ? -m.im : m.im;
-        yi[2 * b + 1] = v.re;
-      }
-      g[3 * k + a].re = df_dot6(xr, yr);
-      g[3 * k + a].im = df_dot6(xi, yi);
-    }
-}
-#endif
 
 // complex sums for the double-float path: lazy (no renormalisation)
 __device__ __forceinline__ Cx<DF> cadd_lazy(Cx<DF> a, Cx<DF> b) { return cx(add_lazy(a.re, b.re), add_lazy(a.im, b.im)); }
@@ -478,17 +447,17 @@ __device__ __forceinline__ void store_rows(char* base, int vh, int s, int row, c
 }
 
 // ------------------------------------------------------------------ epilogues
-// write(): forms and stores the output of one site.  Reducing epilogues with
-// kSplit also offer prepare() (forms the stored words and the reduced value)
-// and commit() (stores them), so that the kernel can publish its block's
-// partial sum before the output stores.  write_rows() is write() for a site
+// write(): forms and stores the output of one site.  Reducing epilogues (kReduce)
+// have prepare() (forms the stored words and the reduced value) and commit()
+// (stores them) in its place, so that the kernel can publish its block's
+// partial sum before the output stores.  write_rows() does both for a site
 // held by two threads (k_hop_rows): a, b are the accumulated spins row and
-// 2 + row; every lane calls it, lanes with ok = false store nothing.
+// 2 + row; every lane calls it, lanes with ok = false store nothing.  The
+// residuals, which are only taken in FP64-class arithmetic, have this form alone.
 // out = coef * H in
 template <int SPO, int COEF>
 struct EpiOut {
   static constexpr bool kReduce = false;
-  static constexpr bool kSplit = false;
   using Packed = int;
   int slot_out;
   int gate;
@@ -522,7 +491,6 @@ struct EpiOut {
 template <int SPO, int SPX, int COEF, bool RED>
 struct EpiXpay {
   static constexpr bool kReduce = RED;
-  static constexpr bool kSplit = RED;
   using Packed = typename Spin<SPO>::Packed;
   int slot_out, slot_x;
   int gate;
@@ -588,7 +556,6 @@ struct EpiXpay {
 template <int SPO, int SPX, int COEF>
 struct EpiXpayDot {
   static constexpr bool kReduce = true;
-  static constexpr bool kSplit = true;
   using Packed = typename Spin<SPO>::Packed;
   int slot_out, slot_x;
   int gate;
@@ -666,28 +633,8 @@ __device__ __forceinline__ void resid_spin(const char* xp, const char* bp, int v
 template <int SPL, int SPH>
 struct EpiResidEO {
   static constexpr bool kReduce = true;
-  static constexpr bool kSplit = false;
-  using Packed = int;
   int gate;
   __host__ double io_bytes() const { return 2.0 * Spin<SPH>::kBytes + Spin<SPL>::kBytes; }
-  template <typename RH>
-  __device__ __forceinline__ void write(const SysDesc& S, int par, int r, int s, Cx<RH> (&acc)[12],
-                                        typename RedT<RH>::type& nrm) const {
-    Cx<RH> x[12], bh[12], rv[12];
-    Spin<SPH>::load(slot_ptr(S, S_X, r, par), S.vh, s, x);
-    Spin<SPH>::load(slot_ptr(S, S_BH, r, par), S.vh, s, bh);
-    const RH k2 = coef<C_PK2, RH>(S);
-    RH n = (RH)0;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      rv[k] = cx(fma(k2, acc[k].re, bh[k].re - x[k].re), fma(k2, acc[k].im, bh[k].im - x[k].im));
-      n = fma(rv[k].re, rv[k].re, fma(rv[k].im, rv[k].im, n));
-    }
-    nrm = to_red(n);
-    Cx<typename Spin<SPL>::R> lo[12];
-    convert12(rv, lo);
-    Spin<SPL>::store(slot_wptr(S, S_R, r, par), S.vh, s, lo);
-  }
   template <typename RH>
   __device__ __forceinline__ void write_rows(const SysDesc& S, int par, int r, int s, int row, Cx<RH> (&a)[3],
                                              Cx<RH> (&b)[3], typename RedT<RH>::type& nrm, bool ok) const {
@@ -707,35 +654,12 @@ struct EpiResidEO {
 template <int SPL, bool STORE_LOW, int SPH>
 struct EpiResidFull {
   static constexpr bool kReduce = true;
-  static constexpr bool kSplit = false;
-  using Packed = int;
   int gate;
   int slot_rt;  // < 0: norm only
   int slot_x;
   int slot_b;
   __host__ double io_bytes() const {
     return 2.0 * Spin<SPH>::kBytes + (slot_rt >= 0 ? Spin<SPH>::kBytes : 0) + (STORE_LOW ? Spin<SPL>::kBytes : 0);
-  }
-  template <typename RH>
-  __device__ __forceinline__ void write(const SysDesc& S, int par, int r, int s, Cx<RH> (&acc)[12],
-                                        typename RedT<RH>::type& nrm) const {
-    Cx<RH> x[12], b[12], rv[12];
-    Spin<SPH>::load(slot_ptr(S, slot_x, r, par), S.vh, s, x);
-    Spin<SPH>::load(slot_ptr(S, slot_b, r, par), S.vh, s, b);
-    const RH kap = coef<C_PK, RH>(S);
-    RH n = (RH)0;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      rv[k] = cx(fma(kap, acc[k].re, b[k].re - x[k].re), fma(kap, acc[k].im, b[k].im - x[k].im));
-      n = fma(rv[k].re, rv[k].re, fma(rv[k].im, rv[k].im, n));
-    }
-    nrm = to_red(n);
-    if (slot_rt >= 0) Spin<SPH>::store(slot_wptr(S, slot_rt, r, par), S.vh, s, rv);
-    if (STORE_LOW) {
-      Cx<typename Spin<SPL>::R> lo[12];
-      convert12(rv, lo);
-      Spin<SPL>::store(slot_wptr(S, S_R, r, par), S.vh, s, lo);
-    }
   }
   template <typename RH>
   __device__ __forceinline__ void write_rows(const SysDesc& S, int par, int r, int s, int row, Cx<RH> (&a)[3],
@@ -968,15 +892,13 @@ __global__ void __launch_bounds__(256, HopOccupancy<SPA>::kMinBlocks)
         hop_mu<2, SPA, LP, C12, SF>(S, in, c, s, r, pin, ulink_own, ulink_nb, mu_stride, acc);
         hop_mu<3, SPA, LP, C12, SF>(S, in, c, s, r, pin, ulink_own, ulink_nb, mu_stride, acc);
       }
-      if constexpr (Epi::kSplit) po = epi.prepare(S, par, r, s, acc, nrm);
+      if constexpr (Epi::kReduce) po = epi.prepare(S, par, r, s, acc, nrm);
       else epi.write(S, par, r, s, acc, nrm);
     }
-    if constexpr (Epi::kSplit) {
+    if constexpr (Epi::kReduce) {
       DW_BLOCK_REDUCE_STORE(nrm, [&] {
         if (valid) epi.commit(S, par, r, s, po);
       })
-    } else if constexpr (Epi::kReduce) {
-      DW_BLOCK_REDUCE(nrm)
     }
   }
 }
@@ -988,7 +910,7 @@ __global__ void __launch_bounds__(256, HopOccupancy<SPA>::kMinBlocks)
 // runs the epilogue.  With one thread per site a 16^3x32 launch has 13 warps
 // per SM, each a serial chain of eight load latencies; four times the warps
 // with a quarter of the chain hide it.  On large lattices the extra pass
-// through shared memory costs more than it gives (the solver's small_lattices
+// through shared memory costs more than it gives (the solver's kSplitSites
 // says where the line lies).
 // Blocks: T sites x RB right-hand sides (T RB <= 128), 4 T RB threads, warps
 // (right-hand side, site group, mu).
@@ -1050,15 +972,13 @@ __global__ void __launch_bounds__(512, 2)
 #pragma unroll
       for (int k = 0; k < 12; ++k)
         acc[k] = acc[k] + cx(mine[(m * 24 + 2 * k) * 32], mine[(m * 24 + 2 * k + 1) * 32]);
-    if constexpr (Epi::kSplit) po = epi.prepare(S, par, r, s, acc, nrm);
+    if constexpr (Epi::kReduce) po = epi.prepare(S, par, r, s, acc, nrm);
     else epi.write(S, par, r, s, acc, nrm);
   }
   if constexpr (Epi::kReduce) {
     const int ntiles = par_mode == 2 ? 2 * S.tpp : S.tpp;
     reduce_block(S, 4 * T, RB, par_mode == 2 ? par * S.tpp + tile : tile, ntiles, nrm, ra, by, [&] {
-      if constexpr (Epi::kSplit) {
-        if (out) epi.commit(S, par, r, s, po);
-      }
+      if (out) epi.commit(S, par, r, s, po);
     });
   }
 }
@@ -1562,7 +1482,7 @@ __global__ void __launch_bounds__(256, 2)
     DW_HOP_PAIR_DIR(2)
     DW_HOP_PAIR_DIR(3)
 #undef DW_HOP_PAIR_DIR
-    if constexpr (Epi::kSplit) {
+    if constexpr (Epi::kReduce) {
       if (v0) po0 = epi.prepare(S, par, r0, s, acc0, nrm[0]);
       if (v1) po1 = epi.prepare(S, par, r1, s, acc1, nrm[1]);
     } else {
@@ -1574,10 +1494,8 @@ __global__ void __launch_bounds__(256, 2)
     const int ntiles = par_mode == 2 ? 2 * S.tpp : S.tpp;
     const int tt = par_mode == 2 ? par * S.tpp + tile : tile;
     reduce_block_n<2>(S, T, RB, tt, ntiles, nrm, ra, by, [&] {
-      if constexpr (Epi::kSplit) {
-        if (v0) epi.commit(S, par, r0, s, po0);
-        if (v1) epi.commit(S, par, r1, s, po1);
-      }
+      if (v0) epi.commit(S, par, r0, s, po0);
+      if (v1) epi.commit(S, par, r1, s, po1);
     });
   }
 }
