@@ -32,19 +32,19 @@ constexpr int kLoopPartials = 2048; // most 32-site tiles of one column: k_finis
 // failure to its whole block, which leaves; the blocks that wait for it run out
 // in turn, and the host solves again with the separate kernels.
 constexpr int kBarrierPolls = 1 << 21;
-__device__ __forceinline__ bool grid_barrier(Flags* f, unsigned& round, int most) {
+__device__ __forceinline__ bool grid_barrier(Flags* f, unsigned& round, int polls) {
   __shared__ int ok_;
   __syncthreads();
   if (gridDim.x == 1) return true;
   round += gridDim.x;
   if (threadIdx.x == 0) {
-    int ok = 1, polls = 0;
+    int ok = 1;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&f->bar_count) : "memory");
     for (;;) {
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&f->bar_count) : "memory");
       if ((int)(v - round) >= 0) break;
-      if (++polls > most) {
+      if (--polls < 0) {
         f->bar_error = 1;
         ok = 0;
         break;
