@@ -1223,8 +1223,8 @@ struct FinPlan {
 // instead of 1024 (launching and draining 32 warps costs more than a longer
 // loop).  With rel.on the last column to finish also sets the condition of the
 // reliable-update node (a separate one-thread kernel would cost about 2 us).
-// Measured at 16^3x32 (512 partials): 4.2 us per launch before, 3.3 now; 24^3x48 with
-// 12 columns of 2592 partials 5.7 and 5.5 us; see k_finish's caller for the rule on
+// Measured at 16^3x32 (both parities, 1024 partials, inside the loop's graph): 4.2 us
+// per launch before, 3.3 now; 24^3x48 with 12 columns of 2592 partials 5.7 and 5.6 us; see k_finish's caller for the rule on
 // the block size.
 constexpr int kFinishThreads = 1024, kFinishThreadsSmall = 256;
 // What the last column of a finishing kernel inside the graph does: on = 1 sets

@@ -1064,7 +1064,8 @@ __device__ __forceinline__ void row_project(const char* in, int vh, int n, int r
 // The FP64 pipe (64 cycles per warp instruction) is the bound, so additions are
 // saved: the backward product's chain starts from g_f and yields A = g_f + g_b
 // at no extra cost, and g_f - g_b = 2 g_f - A is one FMA: 18 instead of 24
-// operations per mu and row, none onto empty sums.
+// operations per mu and row, none onto empty sums.  (Where g_f + g_b is not finite,
+// in the upper spin, g_f - g_b in the lower one is not either.)
 template <bool C12, bool IMAG>
 __device__ __forceinline__ void row_mu(const SysDesc& S, const char* in, const char* own, const char* nbr, int s, int nf,
                                        int nb, int row, int partner, uint32_t cm, uint32_t dm, uint32_t bf, uint32_t bb,
@@ -1405,8 +1406,9 @@ __global__ void __launch_bounds__(512, 1)
 }
 
 // (Since k_hop runs at 64 registers it is the faster of the two on 24^3x48 with 12
-// right-hand sides, 433 against 446 us per application; this one, at 128, stays for
-// the shapes on which the tuner finds it ahead.)
+// right-hand sides, 438 against 461 us per application, although it executes a fifth
+// more instructions; this one, at 128, stays for the shapes on which the tuner finds
+// it ahead.)
 // 16-bit stencil with two right-hand sides per thread: each link is loaded,
 // and with 12-real compression its third row rebuilt, once and applied to
 // both; the two neighbour loads of a direction are in flight together.  Block:

@@ -55,7 +55,8 @@ inline long long parity_work(const std::vector<dw_lattice>& lats, int nrhs) {
 // parities counted where the vectors have both) with all iterations in one
 // kernel (k_cg_loop).  Beyond that its 16 warps per SM lose to the separate
 // kernels: solves with 65536 / 81920 / 131072 sites of a parity, FP16, one kernel
-// 3.16 / 4.54 / 5.25 ms, separate 3.67 / 3.84 / 4.93 ms.
+// 3.16 / 4.54 / 5.25 ms, separate 3.67 / 3.84 / 4.93 ms (nothing was measured
+// between 65536 and 81920).
 // Where blocks of 32 sites and one right-hand side are given (tile, the tuner), the
 // one kernel goes up to kLoopSites too, and up to kLoopSitesFew with at most
 // kFewCols columns, whose partials every block sums.  Solves, one kernel /
@@ -311,9 +312,13 @@ dw_status CG<L, A, C12, H, OP>::build_graph(SolveCacheEntry& ent, int mode, bool
     // A pass of the while node and the test of the if node cost about 4 us each
     // (empty kernels in such a graph: 4.5 us per pass, 8.0 with the if node, 0.6
     // per kernel).  One small column runs four iterations per pass; when one of
-    // them asks for a reliable update the rest of the pass is held.  With larger
-    // grids the held launches cost more than the passes saved, and with several
-    // columns they come too often.
+    // them asks for a reliable update the rest of the pass is held.  Solves, one
+    // iteration per pass / four, ms: 73728 sites of a parity (1152 blocks) FP16
+    // 3.54 / 3.36, FP32 3.56 / 3.37; 331776 (1296 and 2592 blocks) 10.91 / 10.54,
+    // 14.56 / 14.43; 524288 (4096 and 8192) 15.26 / 15.09, 21.16 / 20.78; 1048576
+    // (8192 and 16384) 28.60 / 28.46, 41.52 / 41.37: beyond 2048 blocks four are 0.3
+    // to 2% faster as well, and the line could lie higher.  With several columns
+    // held launches come more often.
     const int per_pass = E.P.ncols == 1 && E.grid(pm).x <= 2048 ? 4 : 1;
     for (int k = 0; k < per_pass; ++k) {
       if (k > 0) {

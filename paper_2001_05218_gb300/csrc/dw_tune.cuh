@@ -113,7 +113,8 @@ BlockShape tune_inner_shape(const std::vector<dw_lattice>& lats, int nrhs, const
   }
   // one-warp blocks only where they are clearly (5%) faster: the update and
   // finishing kernels share the plan and are slower with them (FP32, 16^3x32, the
-  // gradient's normal equations: 22.2 / 19.9 / 20.1 / 20.3 ms with T = 32 / 64 / 128 / 256)
+  // gradient's normal equations: 22.2 / 19.9 / 20.1 / 20.3 ms with T = 32 / 64 / 128 / 256).
+  // The operators, which have no such kernels, read the same record.
   for (int threads : {128, 64})
     for (size_t ci = 0; ci < cand.size(); ++ci)
       if (cand[ci].T * cand[ci].RB == threads && cand[ci].pair == best.pair && best.T * best.RB < 64 &&
