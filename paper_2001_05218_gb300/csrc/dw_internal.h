@@ -116,7 +116,7 @@ cudaError_t device_alloc(char** p, size_t nb);
 enum Refusal {
   REFUSE_LOOP_CAPTURE = 0,  // the cooperative launch, while the loop's graph is captured
   REFUSE_LOOP_START,        // the launch of the instantiated graph
-  REFUSE_LOOP_WAIT,         // every wait of a loop kernel's grid barriers beyond the first look
+  REFUSE_LOOP_WAIT,         // the loop kernel's grid barriers: their count starts one short
   REFUSE_SCRATCH,           // the first attempt of an allocation from the library's pool
   kRefusals
 };

@@ -28,23 +28,22 @@ constexpr int kLoopPartials = 2048; // most 32-site tiles of one column: k_finis
 // (release) and polls it (acquire) until every block of this round has, one trip
 // to L2 and back after the last arrival.  `round` is the count at which this
 // barrier opens; the count runs on through a solve's launches (Flags::bar_base).
-// Every wait is bounded (kBarrierPolls, about a second), then the barrier reports
+// Every wait is bounded: about a second of polls, then the barrier reports
 // failure to its whole block, which leaves; the blocks that wait for it run out
 // in turn, and the host solves again with the separate kernels.
-constexpr int kBarrierPolls = 1 << 21;
-__device__ __forceinline__ bool grid_barrier(Flags* f, unsigned& round, int polls) {
+__device__ __forceinline__ bool grid_barrier(Flags* f, unsigned& round) {
   __shared__ int ok_;
   __syncthreads();
   if (gridDim.x == 1) return true;
   round += gridDim.x;
   if (threadIdx.x == 0) {
-    int ok = 1;
+    int ok = 1, polls = 0;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&f->bar_count) : "memory");
     for (;;) {
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&f->bar_count) : "memory");
       if ((int)(v - round) >= 0) break;
-      if (--polls < 0) {
+      if (++polls > (1 << 21)) {
         f->bar_error = 1;
         ok = 0;
         break;
@@ -201,13 +200,11 @@ __device__ __forceinline__ void loop_hop(const Batch& B, const RedArgs& ra, cons
 }
 
 // B: plan with 32 sites and one right-hand side per block.  rel, loop: the
-// conditions of the reliable-update and the while node.  polls: the most a
-// barrier waits.  MODE: the solver's (even-odd Wilson; the normal equations on
-// both parities; the Laplacian).
+// conditions of the reliable-update and the while node.  MODE: the solver's
+// (even-odd Wilson; the normal equations on both parities; the Laplacian).
 template <int L, int A, bool C12, bool SPLIT, int MODE>
 __global__ void __launch_bounds__(kLoopThreads, 1)
-    k_cg_loop(const __grid_constant__ Batch B, RedArgs ra, unsigned long long rel, unsigned long long loop,
-              int polls) {
+    k_cg_loop(const __grid_constant__ Batch B, RedArgs ra, unsigned long long rel, unsigned long long loop) {
   constexpr bool kNormal = MODE == MODE_NORMAL, kHerm = MODE == MODE_HERM;
   constexpr int OP = kHerm ? OP_LAPLACE : OP_WILSON, PARS = kNormal ? 2 : 1;
   __shared__ ColState cs[kLoopCols];
@@ -235,15 +232,15 @@ __global__ void __launch_bounds__(kLoopThreads, 1)
       if constexpr (kNormal) {
         // t = D p, |t|^2 = p^dag A p; w = D^dag t
         loop_hop<L, C12, SPLIT, false, OP, 2, C_MK>(B, ra, cs, parts, n, 0, S_P, LE_NORM, S_T, S_P, 0);
-        if (!(good = grid_barrier(f, round, polls))) break;
+        if (!(good = grid_barrier(f, round))) break;
         loop_hop<L, C12, SPLIT, true, OP, 2, C_MK>(B, ra, cs, parts, n, 0, S_T, LE_XPAY, S_W, S_T, 0);
       } else {
         // w = Dhat p and |w|^2 (the Laplacian: p^dag w)
         loop_hop<L, C12, SPLIT, false, OP, 1, C_MK2>(B, ra, cs, parts, n, 1, S_P, LE_OUT, S_T, 0, 0);
-        if (!(good = grid_barrier(f, round, polls))) break;
+        if (!(good = grid_barrier(f, round))) break;
         loop_hop<L, C12, SPLIT, false, OP, 1, C_MK2>(B, ra, cs, parts, n, 0, S_T, kHerm ? LE_DOT : LE_NORM, S_W, S_P, 0);
       }
-      if (!(good = grid_barrier(f, round, polls))) break;
+      if (!(good = grid_barrier(f, round))) break;
       column_sums<PARS>(B, ra, ncols, 0, sum);
       if (tid < ncols && cs[tid].active && !form_alpha(cs[tid], sum[tid])) {
         cs[tid].active = 0;
@@ -264,7 +261,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1)
         if (lane == 0) *loop_partial<PARS>(ra, S, t, 1) = to_partial(nrm);
       }
       if (blockIdx.x == 0 && tid == 0) f->late = cs[0].deadline_ns != 0ull && globaltimer_ns() > cs[0].deadline_ns;
-      if (!(good = grid_barrier(f, round, polls))) break;
+      if (!(good = grid_barrier(f, round))) break;
       const bool late = __ldcg(&f->late) != 0;
       column_sums<PARS>(B, ra, ncols, 1, sum);
       if (tid < ncols && cs[tid].active && !count_update(cs[tid], sum[tid], late)) {
@@ -280,9 +277,9 @@ __global__ void __launch_bounds__(kLoopThreads, 1)
     if constexpr (!kNormal && !kHerm) {
       // z = Dhat^dag r, beta
       loop_hop<L, C12, SPLIT, true, OP, 1, C_MK2>(B, ra, cs, parts, n, 1, S_R, LE_OUT, S_T, 0, 0);
-      if (!(good = grid_barrier(f, round, polls))) break;
+      if (!(good = grid_barrier(f, round))) break;
       loop_hop<L, C12, SPLIT, true, OP, 1, C_MK2>(B, ra, cs, parts, n, 0, S_T, LE_NORM, S_Z, S_R, 0);
-      if (!(good = grid_barrier(f, round, polls))) break;
+      if (!(good = grid_barrier(f, round))) break;
       column_sums<PARS>(B, ra, ncols, 0, sum);
       if (tid < ncols && cs[tid].active) form_beta(cs[tid], sum[tid]);
       __syncthreads();
@@ -294,7 +291,7 @@ __global__ void __launch_bounds__(kLoopThreads, 1)
       const SysDesc& S = B.sd[t.si];
       if (t.s < S.vh) update_p_site<L, A>(S, t.par, t.r, t.s, cs[S.col0 + t.r]);
     }
-    if (!(good = grid_barrier(f, round, polls))) break;
+    if (!(good = grid_barrier(f, round))) break;
   }
   // every block holds the same states; the first writes them back
   if (blockIdx.x == 0) {

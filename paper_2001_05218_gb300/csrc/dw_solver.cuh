@@ -182,7 +182,7 @@ struct CG {
     }
     return work <= (P.ncols <= kFewCols ? kLoopSitesFew : kLoopSites);
   }
-  using LoopKernel = void (*)(Batch, RedArgs, unsigned long long, unsigned long long, int);
+  using LoopKernel = void (*)(Batch, RedArgs, unsigned long long, unsigned long long);
   static LoopKernel loop_kernel(const Plan& P, int mode);
   static int loop_grid(const Plan& P, int mode);
   static dw_status launch_loop(const Exec& E, int mode, cudaGraphConditionalHandle rel, cudaGraphConditionalHandle loop);
@@ -267,7 +267,7 @@ dw_status CG<L, A, C12, H, OP>::launch_loop(const Exec& E, int mode, cudaGraphCo
   lc.numAttrs = 1;
   count_launch();
   DW_CUDA(cudaLaunchKernelEx(&lc, loop_kernel(E.P, mode), E.P.B, E.ra(FIN_STORE0), (unsigned long long)rel,
-                             (unsigned long long)loop, refused(REFUSE_LOOP_WAIT) ? 0 : kBarrierPolls));
+                             (unsigned long long)loop));
   return DW_OK;
 }
 
@@ -564,6 +564,7 @@ dw_status CG<L, A, C12, H, OP>::run(const SolveArgs& a) {
   hf.rel_pending = E.P.ncols;
   hf.loops = 0;
   hf.max_loops = a.p.maxiter + 2;
+  if (ent->one && refused(REFUSE_LOOP_WAIT)) hf.bar_count = ~0u;
   cudaEvent_t ev0, ev1;
   DW_CUDA(cudaEventCreate(&ev0));
   DW_CUDA(cudaEventCreate(&ev1));
